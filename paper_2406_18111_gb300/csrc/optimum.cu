@@ -12,12 +12,28 @@
 // an interval of length min_len, min_len + 1, ...  Per string a counter of
 // its intervals in the current set gives "every string at least twice"
 // (no counter at 1) and |T| (counters above 0) at every leaf in O(1).
-// Two cuts that leave the first optimal set in the walk order unchanged:
-// an interval whose string has no second, disjoint occurrence in the window
-// is never tried (every set holding it is infeasible), and a subtree whose
-// coverage bound -- coverage so far plus the positions ahead that some
-// repeatable interval covers -- is below the best coverage found is skipped
-// (none of its sets can reach it).
+// Cuts that leave the first optimal set in the walk order unchanged:
+//   * an interval whose string has no second, disjoint occurrence in the
+//     window is never tried, nor one whose string is not in the set yet and
+//     does not occur again after it (every set below holds it once);
+//   * strings held once need a second interval each: a subtree with fewer
+//     positions ahead than those strings are long is skipped;
+//   * (coverage, intervals) so far plus the best (coverage, intervals) that
+//     repeatable intervals reach from here on, which a recurrence over the
+//     positions gives, bounds every set below (lexicographic order is kept by
+//     adding to both sides); a subtree whose bound does not beat the best set
+//     found before it in the walk, |T| included, is skipped.
+// The bound needs a good set early, and the walk order (uncovered first)
+// meets poor sets first.  So a first walk in the opposite order (intervals
+// before uncovered) finds the optimal value alone, and the second walk, in
+// the order that defines the witness, skips what cannot reach that value.
+//
+// What bounds it: the longest walk of a warp, a serial chain of local-memory
+// accesses (65,536 windows of 20 tokens are one wave).  Nodes of the longest
+// walk in a warp, on those windows at min_len 2: 98,000 with the coverage of
+// the positions ahead as the only bound, 2,900 with the lexicographic bound,
+// 1,800 with the value known as well (both walks counted).  Measured on them:
+// 175 ms before, 6.3 ms with both walks and one warp per block.
 #include <algorithm>
 #include <vector>
 
@@ -34,7 +50,7 @@ constexpr uint64_t kOptLeaves = 1ull << 24;  // largest admissible enumeration
 constexpr uint32_t kOptGuard = 1u << 30;     // node visits after which a walk gives up
 
 template <class T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32)
     k_optimum(const T *__restrict__ tok, const uint32_t *__restrict__ off, uint32_t W, uint32_t m,
               uint32_t *__restrict__ best, uint32_t *__restrict__ wstart, uint32_t *__restrict__ wlen,
               uint32_t *__restrict__ wcount, uint32_t *err) {
@@ -54,109 +70,132 @@ __global__ void __launch_bounds__(128)
       }
     }
     // rep[a] bit L: the length-L string at a occurs again, disjoint from it;
-    // ahead[p]: positions >= p inside some repeatable interval
-    uint32_t rep[kOptMax];
-    for (int a = 0; a < n; ++a) rep[a] = 0;
+    // later[a] bit L: it does so after position a + L - 1
+    uint32_t rep[kOptMax], later[kOptMax];
+    for (int a = 0; a < n; ++a) rep[a] = later[a] = 0;
     for (int a = 0; a < n; ++a)
       for (int b = a + 1; b < n; ++b) {
         int l = 0;
         while (b + l < n && s[a + l] == s[b + l]) ++l;
         const int lim = min(l, b - a);  // disjoint: L <= b - a
-        for (int L = 1; L <= lim; ++L) {
-          rep[a] |= 1u << L;
-          rep[b] |= 1u << L;
-        }
+        const uint32_t lens = (2u << lim) - 2u;
+        rep[a] |= lens;
+        later[a] |= lens;
+        rep[b] |= lens;
       }
-    uint8_t ahead[kOptMax + 1];
-    {
-      uint32_t covered = 0;  // bit i: position i inside a repeatable interval of length >= m
-      for (int a = 0; a < n; ++a)
-        for (int L = (m < 1 ? 1 : (int)m); a + L <= n; ++L)
-          if (rep[a] >> L & 1u) covered |= ((L == 32 ? 0u : (1u << L)) - 1u) << a;
-      ahead[n] = 0;
-      for (int p = n - 1; p >= 0; --p) ahead[p] = (uint8_t)(ahead[p + 1] + ((covered >> p) & 1u));
+    // best (coverage, intervals) of disjoint repeatable intervals at p or
+    // after, coverage in the high byte
+    const int m1 = m < 1 ? 1 : (int)m;
+    uint16_t ahead[kOptMax + 1];
+    ahead[n] = 0;
+    for (int p = n - 1; p >= 0; --p) {
+      int x = ahead[p + 1];
+      for (int L = m1; p + L <= n; ++L)
+        if (rep[p] >> L & 1u) x = max(x, (int)ahead[p + L] + L * 256 + 1);
+      ahead[p] = (uint16_t)x;
     }
     uint8_t cnt[kOptMax * kIdStride];
     for (int i = 0; i < kOptMax * kIdStride; ++i) cnt[i] = 0;
     uint8_t pos[kOptMax + 1], ch[kOptMax + 1];  // ch: 0xff unvisited, 0 uncovered, else interval length
     uint8_t bs[kOptMax], bl[kOptMax];
-    int bk = 0, bcov = -1, bcnt = -1, bdist = 1 << 30;
-    int cov = 0, icnt = 0, singles = 0, distinct = 0;
-    const int m1 = m < 1 ? 1 : (int)m;
-    int d = 0;
-    pos[0] = 0;
-    ch[0] = 0xff;
+    // a set's value: coverage * 256 + intervals, then |T|
+    int bk = 0, bval = -1, bdist = 1 << 30;
+    int vval = -1, vdist = 1 << 30;  // the value the first walk found
     uint32_t guard = 0;
-    while (d >= 0) {
-      if (++guard > kOptGuard) {
-        atomicExch(err, kDevTimeout);
-        break;
-      }
-      const int p = pos[d];
-      if (ch[d] == 0xff) {
-        if (p == n) {  // a complete interval set
-          if (singles == 0 &&
-              (cov > bcov || (cov == bcov && (icnt > bcnt || (icnt == bcnt && distinct < bdist))))) {
-            bcov = cov;
-            bcnt = icnt;
-            bdist = distinct;
-            bk = 0;
-            for (int k = 0; k < d; ++k)
-              if (ch[k]) {
-                bs[bk] = pos[k];
-                bl[bk] = ch[k];
-                ++bk;
-              }
+    for (int walk = 0; walk < 2; ++walk) {
+      int val = 0, singles = 0, sumlen = 0, distinct = 0;  // sumlen: lengths of the strings held once
+      bval = -1;
+      bdist = 1 << 30;
+      int d = 0;
+      pos[0] = 0;
+      ch[0] = 0xff;
+      while (d >= 0) {
+        if (++guard > kOptGuard) {
+          atomicExch(err, kDevTimeout);
+          break;
+        }
+        const int p = pos[d];
+        int L = ch[d];
+        int nx;  // the next choice at p: 0 uncovered, else a length to try from
+        if (L == 0xff) {
+          if (p == n) {  // a complete interval set
+            if (singles == 0 && (val > bval || (val == bval && distinct < bdist))) {
+              bval = val;
+              bdist = distinct;
+              bk = 0;
+              for (int k = 0; walk && k < d; ++k)
+                if (ch[k]) {
+                  bs[bk] = pos[k];
+                  bl[bk] = ch[k];
+                  ++bk;
+                }
+            }
+            --d;
+            continue;
           }
-          --d;
-          continue;
+          const int ub = val + ahead[p];
+          if (sumlen > n - p || ub < bval || (ub == bval && distinct >= bdist) || ub < vval ||
+              (ub == vval && distinct > vdist)) {
+            --d;
+            continue;
+          }
+          nx = walk ? 0 : m1;
+        } else {
+          // back from a child: take the interval of the last choice out
+          if (L) {
+            const int id = sid[p][L] * kIdStride + L;
+            const int c = --cnt[id];
+            if (c == 1) {
+              ++singles;
+              sumlen += L;
+            } else if (c == 0) {
+              --singles;
+              sumlen -= L;
+              --distinct;
+            }
+            val -= L * 256 + 1;
+          }
+          if (!walk && L == 0) {  // uncovered is the first walk's last choice
+            --d;
+            continue;
+          }
+          nx = L ? L + 1 : m1;
         }
-        if (cov + ahead[p] < bcov) {  // cannot reach the best coverage
-          --d;
-          continue;
+        if (nx) {
+          // only strings that can repeat: held already, or found again later
+          while (p + nx <= n &&
+                 !((rep[p] >> nx & 1u) && ((later[p] >> nx & 1u) || cnt[sid[p][nx] * kIdStride + nx])))
+            ++nx;
+          if (p + nx > n) {
+            if (walk) {
+              --d;
+              continue;
+            }
+            nx = 0;
+          }
         }
-        ch[d] = 0;  // position p uncovered
-        pos[d + 1] = (uint8_t)(p + 1);
+        ch[d] = (uint8_t)nx;
+        if (nx) {
+          const int id = sid[p][nx] * kIdStride + nx;
+          const int c = ++cnt[id];
+          if (c == 1) {
+            ++singles;
+            sumlen += nx;
+            ++distinct;
+          } else if (c == 2) {
+            --singles;
+            sumlen -= nx;
+          }
+          val += nx * 256 + 1;
+        }
+        pos[d + 1] = (uint8_t)(p + (nx ? nx : 1));
         ch[d + 1] = 0xff;
         ++d;
-        continue;
       }
-      // back from a child: take the interval of the last choice out, try the next length
-      const int L = ch[d];
-      if (L) {
-        const int id = sid[p][L] * kIdStride + L;
-        const int c = --cnt[id];
-        if (c == 1) ++singles;
-        else if (c == 0) {
-          --singles;
-          --distinct;
-        }
-        cov -= L;
-        --icnt;
-      }
-      int nx = L ? L + 1 : m1;
-      while (p + nx <= n && !(rep[p] >> nx & 1u)) ++nx;  // only strings that can repeat
-      if (p + nx > n) {
-        --d;
-        continue;
-      }
-      ch[d] = (uint8_t)nx;
-      {
-        const int id = sid[p][nx] * kIdStride + nx;
-        const int c = ++cnt[id];
-        if (c == 1) {
-          ++singles;
-          ++distinct;
-        } else if (c == 2) {
-          --singles;
-        }
-        cov += nx;
-        ++icnt;
-      }
-      pos[d + 1] = (uint8_t)(p + nx);
-      ch[d + 1] = 0xff;
-      ++d;
+      vval = bval;
+      vdist = bdist;
     }
+    const int bcov = bval >> 8, bcnt = bval & 255;
     best[3 * w] = (uint32_t)bcov;
     best[3 * w + 1] = (uint32_t)bcnt;
     best[3 * w + 2] = (uint32_t)bdist;
@@ -202,7 +241,7 @@ int optimum_batched(apo_ctx *c, const apo_windows *ws, uint32_t min_len, uint32_
   std::vector<uint32_t> h(W + 1);
   for (uint64_t w = 0; w <= W; ++w) h[w] = (uint32_t)ws->win_off[w];
   APO_CUDA_TRY(cudaMemcpyAsync(off, h.data(), (W + 1) * 4, cudaMemcpyHostToDevice, s));
-  const int threads = 128;
+  const int threads = 32;  // single warps spread evenly: walks differ in length by the window
   const int blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>((W + threads - 1) / threads,
                                                                    (uint64_t)c->num_sms * 64));
   {
