@@ -77,6 +77,7 @@ enum : int {
   kMiscCandUnique = 29,   // candidates left after deduplication
   kMiscRoundTiles = 30,   // tile tickets of a doubling round
   kMiscRoundW = 32,       // 2 x 4 words of consecutive doubling rounds (see build_suffix_array)
+  kMiscSmall = 48,        // 8 words of a small-window call (see small.cu)
   kMiscCount = 64,
 };
 
@@ -96,7 +97,7 @@ enum KernelId : int {
   kKSelOut, kKPatLayout, kKTableInit, kKEndPairs, kKMarkEnds, kKAcFix, kKAcStates,
   kKAcFill, kKDictInsert, kKDictMap, kKSlices, kKMatchOffsets, kKSegScan, kKStarts, kKSparse,
   kKAcNodes, kKAcJump, kKRsTune, kKRpPieces, kKRpNeed, kKRpChain, kKRpAppear, kKRpSelect, kKRpOut,
-  kKOptimum, kKSaDict, kKRound, kKSplit, kKWsb, kKListCompact, kKMinor, kKRsPassKeys, kKAcHalo, kKCount
+  kKOptimum, kKSaDict, kKRound, kKSplit, kKWsb, kKListCompact, kKMinor, kKRsPassKeys, kKAcHalo, kKSmall, kKCount
 };
 extern const char *const kKernelNames[kKCount];
 
@@ -265,6 +266,9 @@ int ensure_side(apo_ctx *c, size_t bytes, cudaStream_t s);
 int check_device_error(apo_ctx *c, cudaStream_t s);
 // Pinned slot that receives the device error word alongside a count read.
 constexpr int kPinnedErr = 15;
+// The pinned buffer: kPinnedWords words for counts, then room for kPinnedOffs
+// words of window offsets.
+constexpr size_t kPinnedWords = 64, kPinnedOffs = 16384;
 int device_error_status(apo_ctx *c, cudaStream_t s);
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -368,6 +372,13 @@ struct BatchOffsets {
 int find_repeats_from_sa(apo_ctx *c, const void *tokens, int token_bytes, const SuffixState &st,
                          const uint32_t *lcp, uint32_t min_len, apo_repeats_out *out,
                          const BatchOffsets *boff, cudaStream_t s);
+
+// Small windows (small.cu): whether a call's windows all take that path, and
+// the call (the workspace is reserved; results and counts as in apo.h).
+bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest);
+int small_find_repeats(apo_ctx *c, const void *tokens, int token_bytes, const uint64_t *win_off, uint32_t windows,
+                       uint32_t longest, const apo_repeats_params *p, apo_repeats_out *out, cudaStream_t s);
+int small_init();
 
 // ---------------------------------------------------------------- hashing
 void launch_hash_tasks(apo_ctx *c, const apo_tasks *t, uint64_t *out, cudaStream_t s);

@@ -136,7 +136,7 @@ const char *const kKernelNames[kKCount] = {
     "ac_states", "ac_fill", "dict_insert", "dict_map", "slices", "match_offsets", "seg_scan",
     "starts", "sparse", "ac_nodes", "ac_jump", "rs_tune", "rp_pieces", "rp_need", "rp_chain",
     "rp_appear", "rp_select", "rp_out", "optimum", "sa_dict", "round", "split", "wsb", "list_compact", "minor",
-    "rs_pass_keys", "ac_halo"};
+    "rs_pass_keys", "ac_halo", "small"};
 
 cudaEvent_t Profiler::get() {
   if (!pool.empty()) {
@@ -237,13 +237,14 @@ int apo_create(apo_ctx **out, int device) {
   int r = APO_OK;
   // (per-device kernel attributes and occupancy; cheap to redo per context)
   if ((r = radix_sort_init()) != APO_OK || (r = suffix_init()) != APO_OK ||
-      (r = repeats_init(optin)) != APO_OK || (r = match_init(c->num_sms)) != APO_OK) {
+      (r = repeats_init(optin)) != APO_OK || (r = match_init(c->num_sms)) != APO_OK ||
+      (r = small_init()) != APO_OK) {
     delete c;
     return r;
   }
   if (cudaMalloc(&c->ps.err, sizeof(uint32_t)) != cudaSuccess ||
       cudaMalloc(&c->ps.counters, kCtrWords * sizeof(uint32_t)) != cudaSuccess ||
-      cudaMallocHost(&c->host_pinned, 256) != cudaSuccess) {
+      cudaMallocHost(&c->host_pinned, (kPinnedWords + kPinnedOffs) * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();
     apo_destroy(c);
     set_error("apo_create: device allocation failed");
@@ -424,6 +425,10 @@ int find_repeats_driver(apo_ctx *c, const void *tokens, int tb, uint64_t total,
     find_repeats_need(n, nwin, &arena_bytes, &lb_words);
     APO_TRY(reserve_workspace(c, arena_bytes, lb_words, s));
   }
+  uint64_t longest = 0;
+  for (uint32_t w = 0; w < nwin; ++w) longest = std::max(longest, win_off[w + 1] - win_off[w]);
+  if (small_windows(c->num_sms, n, nwin, longest))
+    return small_find_repeats(c, tokens, tb, win_off, nwin, (uint32_t)longest, p, out, s);
   SuffixState st;
   st.n = n;
   st.sa = c->arena.take_n<uint32_t>(n);
