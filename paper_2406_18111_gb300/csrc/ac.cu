@@ -1074,48 +1074,45 @@ __global__ void k_lift(const uint32_t *__restrict__ prev_a, uint32_t *__restrict
 
 // Exclusive prefix sum of total[state[x]] over stream positions (the first
 // output slot of each position), decoupled look-back.
-constexpr int kST = 256, kSI = 8, kSTile = kST * kSI;
+// A warp holds kSI rows of 32 consecutive positions (coalesced).
+constexpr int kST = 512, kSI = 8, kSTile = kST * kSI;
 __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restrict__ state,
                                                        const uint32_t *__restrict__ total, uint32_t n,
                                                        uint32_t *__restrict__ off, uint32_t *sum_out,
                                                        uint64_t *status, uint32_t *tile_ctr,
                                                        uint32_t epoch, uint32_t *err) {
-  __shared__ uint32_t s_tile, s_pre;
-  __shared__ uint32_t scr[kST / 32];
-  __shared__ uint32_t sv[kSTile];
-  const int tid = threadIdx.x;
+  __shared__ uint32_t s_tile, s_pre, s_scan[2 * kST / 32];
+  WarpScan<kST / 32> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
   __syncthreads();
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * kSTile;
-  for (int q = tid; q < kSTile; q += kST) sv[q] = base + q < n ? total[state[base + q]] : 0u;
-  __syncthreads();
-  uint32_t run = 0;
+  const uint64_t seg = base + (uint64_t)warp * (kSI * 32) + lane;
+  uint32_t v[kSI], inc[kSI], sum = 0;
 #pragma unroll
-  for (int i = 0; i < kSI; ++i) run += sv[tid * kSI + i];
+  for (int i = 0; i < kSI; ++i) v[i] = seg + i * 32 < n ? state[seg + i * 32] : 0xffffffffu;
+#pragma unroll
+  for (int i = 0; i < kSI; ++i) v[i] = v[i] != 0xffffffffu ? total[v[i]] : 0u;
+#pragma unroll
+  for (int i = 0; i < kSI; ++i) {  // inclusive over the warp's positions
+    inc[i] = sum + warp_inclusive(v[i], OpSum());
+    sum = __shfl_sync(0xffffffffu, inc[i], 31);
+  }
   uint32_t tot;
-  const uint32_t ex = block_exclusive<kST / 32>(run, OpSum(), 0u, scr, &tot);
-  if (tid == 0) {
-    lb_store(&status[t], lb_pack(t == 0 ? kLbInclusive : kLbAggregate, epoch, tot));
-    uint32_t pre = 0;
-    if (t > 0) {
-      pre = lb_exclusive_k<8>(status, 1, t, epoch, OpSum(), 0u, err);
-      lb_store(&status[t], lb_pack(kLbInclusive, epoch, pre + tot));
+  const uint32_t ex = scan.run(sum, OpSum(), &tot);
+  if (warp == 0) {
+    const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
+    if (lane == 0) {
+      s_pre = pre;
+      if (base + kSTile >= n) *sum_out = pre + tot;
     }
-    s_pre = pre;
-    if (base + kSTile >= n) *sum_out = pre + tot;
   }
   __syncthreads();
-  uint32_t r = s_pre + ex;
+  const uint32_t r = s_pre + ex;
 #pragma unroll
-  for (int i = 0; i < kSI; ++i) {  // exclusive offsets back into the tile, then written coalesced
-    const uint32_t v = sv[tid * kSI + i];
-    sv[tid * kSI + i] = r;
-    r += v;
-  }
-  __syncthreads();
-  for (int q = tid; q < kSTile; q += kST)
-    if (base + q < n) off[base + q] = sv[q];
+  for (int i = 0; i < kSI; ++i)
+    if (seg + i * 32 < n) off[seg + i * 32] = r + inc[i] - v[i];
 }
 
 // Pass B: the matches of position x, down the output chain from its state

@@ -70,53 +70,9 @@ __device__ uint32_t lb_exclusive(const uint64_t *status, int stride, uint32_t t,
   return acc;
 }
 
-// The same walk with K predecessor words loaded at once (K loads in flight
-// instead of one dependent load per step).  The words nearer than the first
-// one that is not ready are combined and the walk moves past them; it ends at
-// the first inclusive word.
-template <int K, class Op>
-__device__ uint32_t lb_exclusive_k(const uint64_t *status, int stride, uint32_t t, uint32_t epoch, Op op,
-                                   uint32_t identity, uint32_t *err) {
-  uint32_t acc = identity;
-  long long hi = (long long)t - 1;
-  uint32_t spins = 0;
-  while (hi >= 0) {
-    uint64_t w[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) w[i] = hi - i >= 0 ? lb_load(status + (size_t)(hi - i) * stride) : 0ull;
-    uint32_t part = identity;
-    int used = 0;
-    bool done = false;
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-      if (done || used < i) continue;  // stop at the first word not ready
-      if (hi - i < 0) {
-        done = true;
-        continue;
-      }
-      const uint32_t st = (uint32_t)(w[i] >> 62), ep = (uint32_t)(w[i] >> 32) & 0x3fffffffu;
-      if (ep != epoch || st == kLbNone) continue;
-      part = op((uint32_t)w[i], part);  // tile hi - i precedes the tiles in part
-      used = i + 1;
-      if (st == kLbInclusive) done = true;
-    }
-    acc = op(part, acc);
-    if (done) break;
-    hi -= used;
-    if (used == 0) {
-      if (++spins > kSpinLimit) {
-        atomicExch(err, kDevTimeout);
-        break;
-      }
-      if (spins > 32) __nanosleep(128);
-    }
-  }
-  return acc;
-}
-
-// The same walk by a whole warp, for a commutative operator: lane l reads
-// the word of tile hi - l, so 32 predecessors are combined per step instead
-// of one.  Every lane of the warp must call it; all receive the result.
+// The same walk by a whole warp: lane l reads the word of tile hi - l, so 32
+// predecessors are combined per step instead of one, in index order (the
+// operator need not commute).  Every lane of the warp must call it; all receive the result.
 // The words nearer than the first inclusive one must all be published
 // before the step is taken; otherwise the warp polls them again (bounded as
 // above, then kDevTimeout).
@@ -151,8 +107,11 @@ __device__ uint32_t lb_exclusive_warp(const uint64_t *status, int stride, uint32
     }
     uint32_t v = (lane <= first && j >= 0) ? val : identity;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
-    acc = op(acc, v);
+    for (int o = 1; o < 32; o <<= 1) {  // lane l + o holds an earlier tile than lane l
+      const uint32_t e = __shfl_down_sync(0xffffffffu, v, o);
+      if (lane + o < 32) v = op(e, v);
+    }
+    acc = op(__shfl_sync(0xffffffffu, v, 0), acc);
     if (first < 32) break;
     hi -= 32;
   }
@@ -258,6 +217,39 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, Op op, uint32_t 
   __syncthreads();
   *total = tot;
   return op(pre, wex);
+}
+
+// Exclusive scan over the block's warps of a value that each warp holds
+// uniformly: one barrier (the words alternate between two sets, so a warp
+// may write the next scan's while another still reads this one's).
+template <int NW>
+struct WarpScan {
+  uint32_t *words;  // [2 NW] shared
+  uint32_t par;
+  template <class Op>
+  __device__ __forceinline__ uint32_t run(uint32_t v, Op op, uint32_t *total) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *x = words + (par ? NW : 0);
+    par ^= 1;
+    if (lane == 0) x[warp] = v;
+    __syncthreads();
+    const uint32_t inc = warp_inclusive(lane < NW ? x[lane] : 0u, op);
+    *total = __shfl_sync(0xffffffffu, inc, NW - 1);
+    const uint32_t before = __shfl_sync(0xffffffffu, inc, warp ? warp - 1 : 0);
+    return warp ? before : 0u;
+  }
+};
+
+// Publishes tile t's aggregate v and returns the sum over the tiles before it
+// (the whole warp calls it; every lane gets the sum), then publishes the
+// tile's inclusive prefix.
+__device__ __forceinline__ uint32_t lb_sum_warp(uint64_t *st, uint32_t t, uint32_t v, uint32_t epoch,
+                                                uint32_t *err) {
+  if ((threadIdx.x & 31) == 0) lb_store(&st[t], lb_pack(t == 0 ? kLbInclusive : kLbAggregate, epoch, v));
+  if (t == 0) return 0;
+  const uint32_t p = lb_exclusive_warp(st, 1, t, epoch, OpSum(), 0u, err);
+  if ((threadIdx.x & 31) == 0) lb_store(&st[t], lb_pack(kLbInclusive, epoch, p + v));
+  return p;
 }
 
 }  // namespace apo

@@ -147,8 +147,9 @@ __global__ void k_cand_gen(const uint32_t *__restrict__ sa, const uint32_t *__re
 }
 
 // Order-preserving compaction of the indices k < m with pred(k) (one
-// decoupled look-back sum-scan).
-constexpr int kCT = 256, kCI = 8, kCTile = kCT * kCI;
+// decoupled look-back sum-scan).  A warp holds kCI rows of 32 consecutive
+// indices, so that reads and writes are coalesced.
+constexpr int kCT = 512, kCI = 8, kCTile = kCT * kCI;
 
 struct PredFirstOfRun {  // k starts a run of identical (key, value) pairs (vals == nullptr: keys)
   const uint64_t *keys;
@@ -172,9 +173,10 @@ template <class Pred, class Put>
 __global__ void __launch_bounds__(kCT) k_compact(Pred pred, uint32_t m, const uint32_t *m_dev, uint32_t m_sub,
                                                  Put put, uint32_t *count_out, uint64_t *status,
                                                  uint32_t *tile_ctr, uint32_t epoch, uint32_t *err) {
-  __shared__ uint32_t s_tile, s_pre;
-  __shared__ uint32_t scr[kCT / 32];
-  const int tid = threadIdx.x;
+  __shared__ uint32_t s_tile, s_pre, s_scan[2 * kCT / 32];
+  WarpScan<kCT / 32> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
   if (m_dev) {  // the launch is sized for an upper bound; the count is *m_dev - m_sub
     const uint32_t v = *m_dev;
     m = min(m, v > m_sub ? v - m_sub : 0u);
@@ -184,30 +186,33 @@ __global__ void __launch_bounds__(kCT) k_compact(Pred pred, uint32_t m, const ui
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * kCTile;
   if (t > 0 && base >= m) return;  // past the count (no earlier tile looks at it)
-  const uint64_t e0 = base + (uint64_t)tid * kCI;
-  uint32_t fb = 0;
+  const uint64_t seg = base + (uint64_t)warp * (kCI * 32) + lane;
+  uint32_t bal[kCI], cnt = 0;
+  bool f[kCI];
 #pragma unroll
-  for (int i = 0; i < kCI; ++i)
-    if (e0 + i < m && pred((uint32_t)(e0 + i))) fb |= 1u << i;
-  uint32_t tot;
-  const uint32_t ex = block_exclusive<kCT / 32>(__popc(fb), OpSum(), 0u, scr, &tot);
-  if (tid == 0) {
-    lb_store(&status[t], lb_pack(t == 0 ? kLbInclusive : kLbAggregate, epoch, tot));
-    uint32_t pre = 0;
-    if (t > 0) {
-      pre = lb_exclusive_k<8>(status, 1, t, epoch, OpSum(), 0u, err);
-      lb_store(&status[t], lb_pack(kLbInclusive, epoch, pre + tot));
-    }
-    s_pre = pre;
-    if (base + kCTile >= m) *count_out = pre + tot;
-  }
-  __syncthreads();
-  uint32_t r = s_pre + ex;
+  for (int i = 0; i < kCI; ++i) f[i] = seg + i * 32 < m && pred((uint32_t)(seg + i * 32));
 #pragma unroll
   for (int i = 0; i < kCI; ++i) {
-    if ((fb >> i) & 1u) {
-      if (r < m) put(r, (uint32_t)(e0 + i)); else atomicExch(err, kDevRange);
-      ++r;
+    bal[i] = __ballot_sync(0xffffffffu, f[i]);
+    cnt += __popc(bal[i]);
+  }
+  uint32_t tot;
+  const uint32_t ex = scan.run(cnt, OpSum(), &tot);
+  if (warp == 0) {
+    const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
+    if (lane == 0) {
+      s_pre = pre;
+      if (base + kCTile >= m) *count_out = pre + tot;
+    }
+  }
+  __syncthreads();
+  uint32_t r0 = s_pre + ex;
+#pragma unroll
+  for (int i = 0; i < kCI; ++i) {
+    const uint32_t r = r0 + __popc(bal[i] & lt);
+    r0 += __popc(bal[i]);
+    if ((bal[i] >> lane) & 1u) {
+      if (r < m) put(r, (uint32_t)(seg + i * 32)); else atomicExch(err, kDevRange);
     }
   }
 }
@@ -493,55 +498,54 @@ __global__ void __launch_bounds__(kCT) k_traces(const uint32_t *__restrict__ acc
                                                 uint32_t *__restrict__ svals, uint32_t *tcount,
                                                 uint64_t *status, uint32_t *tile_ctr, uint32_t epoch,
                                                 uint32_t *err) {
-  __shared__ uint32_t s_tile, s_pre;
-  __shared__ uint32_t scr[kCT / 32];
-  const int tid = threadIdx.x;
+  __shared__ uint32_t s_tile, s_pre, s_scan[2 * kCT / 32];
+  WarpScan<kCT / 32> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
   if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
   __syncthreads();
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * kCTile;
-  const uint64_t e0 = base + (uint64_t)tid * kCI;
-  uint32_t fb = 0;
+  const uint64_t seg = base + (uint64_t)warp * (kCI * 32) + lane;
+  uint32_t idx[kCI], len[kCI], bal[kCI], cnt = 0;
+#pragma unroll
+  for (int i = 0; i < kCI; ++i) idx[i] = seg + i * 32 < K ? accidx[seg + i * 32] : 0u;
 #pragma unroll
   for (int i = 0; i < kCI; ++i) {
-    const uint64_t q = e0 + i;
-    if (q < K) {
-      const uint32_t k = accidx[q];
-      bool f = q == 0;
-      if (!f) {
-        const uint32_t kp = accidx[q - 1];
-        f = cl[k] != cl[kp] || cid[k] != cid[kp];
-      }
-      if (f) fb |= 1u << i;
+    const uint64_t q = seg + i * 32;
+    bool f = q == 0 && K > 0;
+    len[i] = q < K ? cl[idx[i]] : 0u;
+    if (q < K && q > 0) {
+      const uint32_t kp = accidx[q - 1];
+      f = len[i] != cl[kp] || cid[idx[i]] != cid[kp];
     }
+    bal[i] = __ballot_sync(0xffffffffu, f);
+    cnt += __popc(bal[i]);
   }
   uint32_t tot;
-  const uint32_t ex = block_exclusive<kCT / 32>(__popc(fb), OpSum(), 0u, scr, &tot);
-  if (tid == 0) {
-    lb_store(&status[t], lb_pack(t == 0 ? kLbInclusive : kLbAggregate, epoch, tot));
-    uint32_t pre = 0;
-    if (t > 0) {
-      pre = lb_exclusive_k<8>(status, 1, t, epoch, OpSum(), 0u, err);
-      lb_store(&status[t], lb_pack(kLbInclusive, epoch, pre + tot));
+  const uint32_t ex = scan.run(cnt, OpSum(), &tot);
+  if (warp == 0) {
+    const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
+    if (lane == 0) {
+      s_pre = pre;
+      if (base + kCTile >= K) *tcount = pre + tot;
     }
-    s_pre = pre;
-    if (base + kCTile >= K) *tcount = pre + tot;
   }
   __syncthreads();
-  uint32_t run = s_pre + ex;  // trace starts before element e0
+  uint32_t run = s_pre + ex;  // trace starts before the warp's row
 #pragma unroll
   for (int i = 0; i < kCI; ++i) {
-    const uint64_t q = e0 + i;
+    const uint64_t q = seg + i * 32;
+    const bool f = (bal[i] >> lane) & 1u;
+    const uint32_t tr = run + __popc(bal[i] & lt) + (f ? 1u : 0u) - 1;  // index of this candidate's trace
+    run += __popc(bal[i]);
     if (q < K) {
-      const uint32_t k = accidx[q];
-      const bool f = (fb >> i) & 1u;
-      run += f;
-      const uint32_t tr = run - 1;  // index of this candidate's trace
+      const uint32_t st = cs[idx[i]];
       if (f) {
-        tl[tr] = cl[k];
-        ts[tr] = cs[k];
+        tl[tr] = len[i];
+        ts[tr] = st;
       }
-      skeys[q] = ((uint64_t)cs[k] << 32) | cl[k];
+      skeys[q] = ((uint64_t)st << 32) | len[i];
       svals[q] = tr;
     }
   }

@@ -85,27 +85,6 @@ struct SmallArgs {
 
 __device__ __forceinline__ int sm_bits(uint32_t v) { return v ? 32 - __clz(v) : 0; }
 
-// Exclusive scan over the block's warps of a value that each warp holds
-// uniformly: one barrier (the words alternate between two sets, so a warp
-// may write the next scan's while another still reads this one's).
-template <int NW>
-struct WarpScan {
-  uint32_t *words;  // [2 NW] shared
-  uint32_t par;
-  template <class Op>
-  __device__ __forceinline__ uint32_t run(uint32_t v, Op op, uint32_t *total) {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *x = words + (par ? NW : 0);
-    par ^= 1;
-    if (lane == 0) x[warp] = v;
-    __syncthreads();
-    const uint32_t inc = warp_inclusive(lane < NW ? x[lane] : 0u, op);
-    *total = __shfl_sync(0xffffffffu, inc, NW - 1);
-    const uint32_t before = __shfl_sync(0xffffffffu, inc, warp ? warp - 1 : 0);
-    return warp ? before : 0u;
-  }
-};
-
 // One stable LSD radix pass after another over bits [lo, hi) of buf[0, cnt)
 // (and of the values in vbuf).  A thread keeps its keys in registers between
 // the read and the scatter, so the sort is in place.  Digits in which `diff`

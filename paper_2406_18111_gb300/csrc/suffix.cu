@@ -102,23 +102,9 @@ __device__ __forceinline__ uint32_t level_rank(const uint8_t *__restrict__ fin, 
   return f <= L ? rank[j] : snap[j];
 }
 
-// Decoupled look-back: lb_publish stores the tile's aggregate, lb_sum_warp
-// publishes it and resolves the sum over tiles < t with one warp, then stores
-// the tile's inclusive prefix.  A tile should resolve right after it
-// publishes: a walk back only ends at an inclusive prefix, so tiles that
-// resolve late make their successors' walks long.
-__device__ __forceinline__ void lb_publish(uint64_t *st, uint32_t t, uint32_t v, uint32_t epoch) {
-  lb_store(&st[t], lb_pack(t == 0 ? kLbInclusive : kLbAggregate, epoch, v));
-}
-// Every lane of the warp calls it; all get the prefix.
-__device__ __forceinline__ uint32_t lb_sum_warp(uint64_t *st, uint32_t t, uint32_t v, uint32_t epoch,
-                                                uint32_t *err) {
-  if ((threadIdx.x & 31) == 0) lb_publish(st, t, v, epoch);
-  if (t == 0) return 0;
-  const uint32_t p = lb_exclusive_warp(st, 1, t, epoch, OpSum(), 0u, err);
-  if ((threadIdx.x & 31) == 0) lb_store(&st[t], lb_pack(kLbInclusive, epoch, p + v));
-  return p;
-}
+// Tiles publish and resolve their look-backs as early as they can: a walk
+// back only ends at an inclusive prefix, so tiles that resolve late make
+// their successors' walks long.
 
 // ---------------------------------------------------------------- settling sorted groups
 // Sorted (key, suffix) pairs -> groups of equal keys.  Every suffix gets its
@@ -134,7 +120,13 @@ __device__ __forceinline__ uint32_t lb_sum_warp(uint64_t *st, uint32_t t, uint32
 //   hole.
 // Decoupled look-backs: the last group start (max) and, for kBig false, the
 // list position (sum).
-constexpr int kST = 256, kSI = 4, kSTile = kST * kSI;
+//
+// A warp holds kSI rows of 32 consecutive elements, so that every read and
+// every list write is coalesced and the flags of a row are one ballot.  What
+// bounds it: the scattered writes by suffix, and the wait for the look-back,
+// whose walk is as long as there are tiles in flight -- hence tiles of 4,096
+// elements (with 1,024 the blocks spent most of their time at that barrier).
+constexpr int kST = 512, kSI = 8, kSTile = kST * kSI;
 
 template <bool kBig>
 __global__ void __launch_bounds__(kST) k_split(
@@ -145,119 +137,121 @@ __global__ void __launch_bounds__(kST) k_split(
     uint8_t *__restrict__ fin, uint32_t *__restrict__ nid, uint32_t *__restrict__ nhd, uint32_t list_cap,
     uint32_t *count_out, uint32_t n, uint64_t *st_max, uint64_t *st_sum, uint32_t *tile_ctr, uint32_t epoch,
     uint32_t *err, int id_bits) {
-  __shared__ uint64_t sk[kSTile + 2];  // key of element base - 1 + q (without the suffix bits)
-  __shared__ uint32_t sv[kSTile];
-  __shared__ uint32_t s_tile, s_pmax, s_psum;
-  __shared__ uint32_t scr[kST / 32];
-  const int tid = threadIdx.x;
+  constexpr int NW = kST / 32;
+  __shared__ uint32_t s_tile, s_pmax, s_psum, s_scan[2 * NW];
+  WarpScan<NW> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
   const uint32_t N = n_dev ? min(ub, *n_dev) : ub;
   if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
   __syncthreads();
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * kSTile;
   if (base >= N) return;  // past the device-side count: no later tile looks at it
-  const uint32_t cnt = (N - base) < (uint64_t)kSTile ? (uint32_t)(N - base) : (uint32_t)kSTile;
+  const uint64_t seg = base + (uint64_t)warp * (kSI * 32);  // the warp's first element
   // id_bits > 0: the suffix is the key's low id_bits bits (keys-only sort)
-  const uint64_t idmask = id_bits ? (1ull << id_bits) - 1 : 0ull;
-  for (uint32_t q = tid; q < cnt + 2; q += kST) {
-    const long long g = (long long)base - 1 + q;
-    const uint64_t kv = (g >= 0 && g < (long long)N) ? keys[g] : 0;
-    sk[q] = kv >> id_bits;
-    if (id_bits && q >= 1 && q <= cnt) sv[q - 1] = (uint32_t)(kv & idmask);
-  }
-  if (!id_bits)
-    for (uint32_t q = tid; q < cnt; q += kST) sv[q] = vals[base + q];
-  __syncthreads();
-
-  const uint32_t e0 = tid * kSI;
-  uint32_t hb = 0;  // bit i: element e0 + i starts a group (bit kSI: the element after)
+  const uint32_t idmask = id_bits ? (uint32_t)((1ull << id_bits) - 1) : 0u;
+  uint64_t k[kSI];  // keys without the suffix bits
+  uint32_t id[kSI];
 #pragma unroll
-  for (int i = 0; i <= kSI; ++i) {
-    const uint32_t local = e0 + i;
-    if (local <= cnt) {
-      const uint64_t g = base + local;
-      if (g == 0 || g == N || sk[local + 1] != sk[local]) hb |= 1u << i;
+  for (int j = 0; j < kSI; ++j) {
+    const uint64_t g = seg + j * 32 + lane;
+    k[j] = g < N ? keys[g] : 0;
+    id[j] = g < N && !id_bits ? vals[g] : 0u;
+  }
+  uint64_t edge = 0;  // lane 0: the key before the warp's elements; lane 31: the one after them
+  if (lane == 0 && seg > 0 && seg < N) edge = keys[seg - 1] >> id_bits;
+  if (lane == 31 && seg + kSI * 32 < N) edge = keys[seg + kSI * 32] >> id_bits;
+#pragma unroll
+  for (int j = 0; j < kSI; ++j) {
+    if (id_bits) {
+      id[j] = (uint32_t)k[j] & idmask;
+      k[j] >>= id_bits;
     }
   }
-  uint32_t tmax = 0, tcnt = 0;
-  bool thead = false;
+  // row j's ballot: elements that start a group (also the first one past N);
+  // wmax: 1 + the warp's last start
+  uint32_t hb[kSI + 1], wmax = 0, wcnt = 0;
 #pragma unroll
-  for (int i = 0; i < kSI; ++i) {
-    if (e0 + i < cnt) {
-      const bool h = (hb >> i) & 1u;
-      if (h) {
-        tmax = (uint32_t)(base + e0 + i);
-        thead = true;
-      }
-      if (!(h && ((hb >> (i + 1)) & 1u))) ++tcnt;
-    }
+  for (int j = 0; j < kSI; ++j) {
+    const uint64_t g = seg + j * 32 + lane;
+    uint64_t prev = __shfl_up_sync(0xffffffffu, k[j], 1);
+    const uint64_t carry = j ? __shfl_sync(0xffffffffu, k[j - (j ? 1 : 0)], 31) : edge;
+    if (lane == 0) prev = carry;
+    hb[j] = __ballot_sync(0xffffffffu, g < N ? (g == 0 || prev != k[j]) : g == N);
+    const uint32_t in = hb[j] & __ballot_sync(0xffffffffu, g < N);
+    if (in) wmax = (uint32_t)(seg + j * 32) + (31 - __clz(in)) + 1;
   }
-  uint32_t tot_max, tot_sum;
-  const uint32_t ex_max = block_exclusive<kST / 32>(tmax, OpMax(), 0u, scr, &tot_max);
-  const uint32_t ex_sum = kBig ? 0u : block_exclusive<kST / 32>(tcnt, OpSum(), 0u, scr, &tot_sum);
-  const int any_head = __syncthreads_or(thead);
-  if (tid < 32) {
-    const bool incl = t == 0 || any_head;  // a tile with a group start knows its maximum
-    if (tid == 0) lb_store(&st_max[t], lb_pack(incl ? kLbInclusive : kLbAggregate, epoch, tot_max));
-    uint32_t pm = 0;
-    if (t > 0) pm = lb_exclusive_warp(st_max, 1, t, epoch, OpMax(), 0u, err);
-    if (tid == 0) {
+  {
+    const uint64_t g = seg + kSI * 32;  // the first element after the warp's
+    hb[kSI] = __ballot_sync(0xffffffffu, lane == 31 && (g < N ? edge != k[kSI - 1] : g == N)) ? 1u : 0u;
+  }
+  // not alone: the element does not start a group, or the next one does not
+  uint32_t keep[kSI];
+#pragma unroll
+  for (int j = 0; j < kSI; ++j) {
+    const uint32_t nxt = (hb[j] >> 1) | (hb[j + 1] << 31);
+    keep[j] = ~(hb[j] & nxt) & __ballot_sync(0xffffffffu, seg + j * 32 + lane < N);
+    wcnt += __popc(keep[j]);
+  }
+  uint32_t tot_max, tot_sum = 0;
+  uint32_t hq = scan.run(wmax, OpMax(), &tot_max);
+  uint32_t rs = kBig ? 0u : scan.run(wcnt, OpSum(), &tot_sum);
+  if (warp == 0) {
+    const bool incl = t == 0 || tot_max;  // a tile with a group start knows its maximum
+    if (lane == 0) lb_store(&st_max[t], lb_pack(incl ? kLbInclusive : kLbAggregate, epoch, tot_max));
+    const uint32_t pm = t > 0 ? lb_exclusive_warp(st_max, 1, t, epoch, OpMax(), 0u, err) : 0u;
+    if (lane == 0) {
       if (!incl) lb_store(&st_max[t], lb_pack(kLbInclusive, epoch, max(pm, tot_max)));
       s_pmax = pm;
     }
-  } else if (!kBig && tid < 64) {
+  } else if (!kBig && warp == 1) {
     const uint32_t ps = lb_sum_warp(st_sum, t, tot_sum, epoch, err);
-    if (tid == 32) {
+    if (lane == 0) {
       s_psum = ps;
-      if (finals && base + cnt == N) *count_out = ps + tot_sum;
+      if (finals && base + kSTile >= N) *count_out = ps + tot_sum;
     }
   }
   __syncthreads();
-  uint32_t hq = max(s_pmax, ex_max);  // index of the current group's first element
-  uint32_t rs = kBig ? 0u : s_psum + ex_sum;
+  hq = max(s_pmax, hq);  // 1 + index of the last group start before the warp's elements
+  if (!kBig) rs += s_psum;
 #pragma unroll
-  for (int i = 0; i < kSI; ++i) {
-    const uint32_t local = e0 + i;
-    if (local >= cnt) break;
-    const bool h = (hb >> i) & 1u;
-    const uint32_t q = (uint32_t)(base + local);
-    if (h) hq = q;
-    const uint32_t id = sv[local];
-    uint32_t slot = q, head = hq, at = 0;
+  for (int j = 0; j < kSI; ++j) {
+    const uint64_t g = seg + j * 32 + lane;
+    const uint32_t row = (uint32_t)(seg + j * 32), mine = hb[j] & le;
+    const uint32_t hd = (mine ? row + (31 - __clz(mine)) + 1 : hq) - 1;  // index of the group's first element
+    if (hb[j]) hq = row + (31 - __clz(hb[j])) + 1;  // (past N only behind the last element)
+    const uint32_t at0 = rs + __popc(keep[j] & lt);
+    rs += __popc(keep[j]);
+    if (g >= N) continue;
+    const uint32_t q = (uint32_t)g;
+    uint32_t slot = q, head = hd, at = at0;
     if (kBig) {
-      const uint32_t o = (uint32_t)(sk[local + 1] >> ord_shift);
+      const uint32_t o = (uint32_t)(k[j] >> ord_shift);
       if (o >= bg_cap) {
         atomicExch(err, kDevRange);
         continue;
       }
       const uint32_t hs = bg_head[o], bo = bg_off[o];
       slot = hs + (q - bo);
-      head = hs + (hq - bo);
+      head = hs + (hd - bo);
       at = bg_pos[o] + (q - bo);
     }
-    if (id >= n || slot >= n || (kBig && at >= list_cap)) {
+    const bool alone = finals && !((keep[j] >> lane) & 1u);
+    if (id[j] >= n || slot >= n || (finals && (kBig || !alone) && at >= list_cap)) {
       atomicExch(err, kDevRange);
       continue;
     }
-    const bool alone = finals && h && ((hb >> (i + 1)) & 1u);
-    if (!alone) snap[id] = head;  // (a final suffix's level rank is its rank[])
+    if (!alone) snap[id[j]] = head;  // (a final suffix's level rank is its rank[])
     if (!finals) continue;
     if (alone) {
-      sa[slot] = id;
-      rank[id] = slot;
-      fin[id] = (uint8_t)level;
+      sa[slot] = id[j];
+      rank[id[j]] = slot;
+      fin[id[j]] = (uint8_t)level;
       if (kBig) nhd[at] = kHole;
-    } else if (kBig) {
-      nid[at] = id;
-      nhd[at] = head;
     } else {
-      if (rs < list_cap) {
-        nid[rs] = id;
-        nhd[rs] = head;
-      } else {
-        atomicExch(err, kDevRange);
-      }
-      ++rs;
+      nid[at] = id[j];
+      nhd[at] = head;
     }
   }
 }
@@ -938,34 +932,38 @@ __global__ void __launch_bounds__(kRdThreads, 4) k_round(const RoundArgs a) {
 
 // The holed next list (entries settled in place, holes where a suffix became
 // final) -> the dense next list, order kept; its length lands in *count_out.
-constexpr int kLcT = 256, kLcI = 8, kLcTile = kLcT * kLcI;
+// A warp holds kLcI rows of 32 consecutive entries (coalesced both ways).
+constexpr int kLcT = 512, kLcI = 8, kLcTile = kLcT * kLcI;
 __global__ void __launch_bounds__(kLcT) k_list_compact(const uint32_t *__restrict__ hid,
                                                        const uint32_t *__restrict__ hhd, uint32_t ub,
                                                        const uint32_t *__restrict__ A_dev,
                                                        uint32_t *__restrict__ nid, uint32_t *__restrict__ nhd,
                                                        uint32_t n, uint32_t *count_out, uint64_t *status,
                                                        uint32_t *tile_ctr, uint32_t epoch, uint32_t *err) {
-  __shared__ uint32_t s_tile, s_pre;
-  __shared__ uint32_t scr[kLcT / 32];
-  const int tid = threadIdx.x;
+  __shared__ uint32_t s_tile, s_pre, s_scan[2 * kLcT / 32];
+  WarpScan<kLcT / 32> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
   if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
   const uint32_t A = min(ub, *A_dev);
   __syncthreads();
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * kLcTile;
   if (base >= A) return;
-  uint32_t hd[kLcI], cnt = 0;
+  const uint64_t seg = base + (uint64_t)warp * (kLcI * 32) + lane;
+  uint32_t hd[kLcI], id[kLcI], cnt = 0;
+#pragma unroll
+  for (int i = 0; i < kLcI; ++i) hd[i] = seg + i * 32 < A ? hhd[seg + i * 32] : kHole;
 #pragma unroll
   for (int i = 0; i < kLcI; ++i) {
-    const uint64_t k = base + (uint64_t)tid * kLcI + i;
-    hd[i] = k < A ? hhd[k] : kHole;
-    cnt += hd[i] != kHole;
+    id[i] = hd[i] != kHole ? hid[seg + i * 32] : 0u;
+    cnt += __popc(__ballot_sync(0xffffffffu, hd[i] != kHole));
   }
   uint32_t tot;
-  const uint32_t ex = block_exclusive<kLcT / 32>(cnt, OpSum(), 0u, scr, &tot);
-  if (tid < 32) {
+  const uint32_t ex = scan.run(cnt, OpSum(), &tot);
+  if (warp == 0) {
     const uint32_t p = lb_sum_warp(status, t, tot, epoch, err);
-    if (tid == 0) {
+    if (lane == 0) {
       s_pre = p;
       if (base + kLcTile >= A) *count_out = p + tot;
     }
@@ -974,15 +972,16 @@ __global__ void __launch_bounds__(kLcT) k_list_compact(const uint32_t *__restric
   uint32_t rs = s_pre + ex;
 #pragma unroll
   for (int i = 0; i < kLcI; ++i) {
+    const uint32_t b = __ballot_sync(0xffffffffu, hd[i] != kHole);
+    const uint32_t r = rs + __popc(b & lt);
+    rs += __popc(b);
     if (hd[i] == kHole) continue;
-    const uint64_t k = base + (uint64_t)tid * kLcI + i;
-    if (rs < n) {
-      nid[rs] = hid[k];
-      nhd[rs] = hd[i];
+    if (r < n) {
+      nid[r] = id[i];
+      nhd[r] = hd[i];
     } else {
       atomicExch(err, kDevRange);
     }
-    ++rs;
   }
 }
 
