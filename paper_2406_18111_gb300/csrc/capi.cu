@@ -368,14 +368,30 @@ int apo_hash_tasks(apo_ctx *c, const apo_tasks *t, uint64_t *tokens_out, void *s
 namespace apo {
 namespace drv {
 
-__global__ void k_fill_windows(const uint32_t *__restrict__ off, uint32_t count, uint32_t *wid,
-                               uint32_t *wend) {
-  for (uint32_t w = blockIdx.x; w < count; w += gridDim.x) {
-    const uint32_t a = off[w], b = off[w + 1];
-    for (uint32_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-      wid[i] = w;
-      wend[i] = b;
-    }
+// wid[i], wend[i]: the window of position i and that window's end.  A block
+// fills kFillTile consecutive positions, so that a long window's positions
+// are spread over many blocks (one block per window took 100 us for 512
+// windows of 1,024 to 262,144 tokens).
+constexpr uint32_t kFillTile = 4096;
+__device__ __forceinline__ uint32_t window_of(const uint32_t *__restrict__ off, uint32_t lo, uint32_t hi, uint32_t i) {
+  while (lo < hi) {  // the last window in [lo, hi] that starts at or before i (empty windows before it share its start)
+    const uint32_t mid = lo + (hi - lo + 1) / 2;
+    if (off[mid] <= i) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+__global__ void __launch_bounds__(256) k_fill_windows(const uint32_t *__restrict__ off, uint32_t count, uint32_t n,
+                                                      uint32_t *__restrict__ wid, uint32_t *__restrict__ wend) {
+  __shared__ uint32_t s_w[2];
+  const uint32_t base = blockIdx.x * kFillTile, last = min(n - base, kFillTile) - 1 + base;
+  if (threadIdx.x < 2) s_w[threadIdx.x] = window_of(off, 0, count - 1, threadIdx.x ? last : base);
+  __syncthreads();
+  const uint32_t w0 = s_w[0], w1 = s_w[1];
+  for (uint32_t i = base + threadIdx.x; i <= last; i += 256) {
+    const uint32_t w = w0 == w1 ? w0 : window_of(off, w0, w1, i);
+    wid[i] = w;
+    wend[i] = off[w + 1];
   }
 }
 
@@ -460,7 +476,7 @@ int find_repeats_driver(apo_ctx *c, const void *tokens, int tb, uint64_t total,
     }
     {
       Launch lp_(c, kKInitKeys, n, s);
-      k_fill_windows<<<std::min<uint32_t>(nwin, 4096), 256, 0, s>>>(off, nwin, wid, wend);
+      k_fill_windows<<<ceil_div(n, kFillTile), 256, 0, s>>>(off, nwin, n, wid, wend);
     }
     if (!capturing(c)) APO_CUDA_TRY(cudaStreamSynchronize(s));  // h goes out of scope
     st.win.wid = wid;

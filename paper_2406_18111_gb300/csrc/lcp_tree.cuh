@@ -53,6 +53,41 @@ __device__ __forceinline__ long long prev_less(const MinTree &T, uint32_t k, uin
   return -1;
 }
 
+// prev_less for the 32 consecutive entries k = base + lane of a warp (base a
+// multiple of 32; the whole warp calls it; v = entry k, 0 past the array; l <=
+// v).  Meaningful for lanes with `want`.  Within the block the entries are in
+// the warp's registers: every lane follows links to the previous smaller
+// entry, which the lanes shorten for each other (a link of a link skips
+// nothing that is smaller); a lane that finds none walks the levels above.
+__device__ __forceinline__ long long prev_less_warp(const MinTree &T, uint32_t base, uint32_t v, uint32_t l,
+                                                    bool want, uint32_t *err) {
+  const int lane = threadIdx.x & 31;
+  int link = lane - 1;  // entries link + 1 .. lane - 1 are >= v
+  bool open = link >= 0;
+  while (__any_sync(0xffffffffu, open)) {
+    const uint32_t y = __shfl_sync(0xffffffffu, v, link & 31);
+    const int next = __shfl_sync(0xffffffffu, link, link & 31);
+    if (open) {
+      if (y >= v) link = next;
+      else open = false;
+      if (link < 0) open = false;
+    }
+  }
+  int f = link;
+  open = want && f >= 0 && l < v;  // a truncated length: on to the first entry below it
+  while (__any_sync(0xffffffffu, open)) {
+    const uint32_t y = __shfl_sync(0xffffffffu, v, f & 31);
+    const int next = __shfl_sync(0xffffffffu, link, f & 31);
+    if (open) {
+      if (y >= l) f = next;
+      else open = false;
+      if (f < 0) open = false;
+    }
+  }
+  if (!want) return -1;
+  return f >= 0 ? (long long)base + f : base ? prev_less(T, base, l, err) : -1;
+}
+
 // Builds the levels above `lcp` (n entries) from the context's arena.
 int build_min_tree(apo_ctx *c, const uint32_t *lcp, uint32_t n, MinTree *T, cudaStream_t s);
 

@@ -69,80 +69,106 @@ __device__ __forceinline__ void pair_cand(uint32_t s1, uint32_t s2, uint32_t p, 
   }
 }
 
-__global__ void k_cand_gen(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ lcp,
-                           uint32_t n, uint32_t min_len, MinTree T, int bi, int bl, uint32_t lmax, int ks,
-                           Windows W, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                           uint32_t *count, uint32_t *err, uint32_t *__restrict__ hist, int hist_bits) {
+// A block takes kGenT * kGenI pairs at a time and reserves their entries with
+// one addition to the count (one per warp queued on the one address).
+constexpr int kGenT = 256, kGenI = 4;
+__global__ void __launch_bounds__(kGenT) k_cand_gen(
+    const uint32_t *__restrict__ sa, const uint32_t *__restrict__ lcp, uint32_t n, uint32_t min_len, MinTree T, int bi,
+    int bl, uint32_t lmax, int ks, Windows W, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
+    uint32_t *count, uint32_t *err, uint32_t *__restrict__ hist, int hist_bits) {
   // the sort's first digit place (the key's lowest hist_bits bits when the
   // key holds the start, else the value's): counted here for the sort
   __shared__ uint32_t sh[512];
+  __shared__ uint32_t s_base, s_scan[2 * kGenT / 32];
+  WarpScan<kGenT / 32> scan{s_scan, 0};
   const uint32_t hmask = (1u << hist_bits) - 1;
-  for (uint32_t d = threadIdx.x; d <= hmask; d += blockDim.x) sh[d] = 0;
+  for (uint32_t d = threadIdx.x; d <= hmask; d += kGenT) sh[d] = 0;
   __syncthreads();
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t base = blockIdx.x * blockDim.x; base < n - 1; base += stride) {
-    const uint32_t k = base + threadIdx.x;
-    bool ok = false, ok_b = false;
-    uint32_t l = 0, a = 0, b = 0;
-    if (k < n - 1) {
-      pair_cand(sa[k], sa[k + 1], lcp[k], &l, &a, &b);
-      ok = l >= min_len && l > 0;
-      // pair k + 1's first candidate is often this pair's second one (equal
-      // LCPs along a run of the SA): leave it to pair k + 1
-      ok_b = ok;
-      if (ok && k + 1 < n - 1) {
-        uint32_t l2, a2, b2;
-        pair_cand(sa[k + 1], sa[k + 2], lcp[k + 1], &l2, &a2, &b2);
-        if (l2 == l && a2 == b) ok_b = false;
+  const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
+  const uint64_t stride = (uint64_t)gridDim.x * kGenT * kGenI;
+  for (uint64_t base0 = (uint64_t)blockIdx.x * kGenT * kGenI; base0 < n - 1; base0 += stride) {
+    uint64_t key[kGenI];
+    uint32_t a[kGenI], b[kGenI], okb[kGenI], ok_bb[kGenI], cnt = 0;  // the rows' ballots
+#pragma unroll
+    for (int i = 0; i < kGenI; ++i) {
+      const uint64_t row = base0 + i * kGenT + (threadIdx.x & ~31u);
+      const uint64_t k64 = row + lane;
+      const uint32_t k = (uint32_t)k64;
+      bool ok = false, ok_b = false;
+      uint32_t l = 0, p = 0;
+      a[i] = b[i] = 0;
+      if (k64 < n - 1) {
+        const uint32_t s1 = sa[k + 1];
+        p = lcp[k];
+        pair_cand(sa[k], s1, p, &l, &a[i], &b[i]);
+        ok = l >= min_len && l > 0;
+        // pair k + 1's first candidate is often this pair's second one (equal
+        // LCPs along a run of the SA): leave it to pair k + 1
+        ok_b = ok;
+        if (ok && k + 1 < n - 1) {
+          uint32_t l2, a2, b2;
+          pair_cand(s1, sa[k + 2], lcp[k + 1], &l2, &a2, &b2);
+          if (l2 == l && a2 == b[i]) ok_b = false;
+        }
+      }
+      key[i] = 0;
+      if (__any_sync(0xffffffffu, ok)) {
+        const long long j = prev_less_warp(T, (uint32_t)row, p, l, ok, err);
+        if (ok) {
+          // with several windows, the id and the start are relative to the
+          // window (its suffixes occupy a contiguous SA range starting at its
+          // offset), which keeps the key and value digits to the longest window
+          // (the pair's SA slots and suffixes lie in the same window: its id is
+          // read at slot k, next to the other threads' reads)
+          const uint32_t w = win_id(W, k), wbase = W.off_dev ? W.off_dev[w] : 0u;
+          const uint32_t wlen = (W.off_dev ? W.off_dev[w + 1] : n) - wbase;
+          if (a[i] < wbase || b[i] < wbase || a[i] - wbase + (uint64_t)l > wlen ||
+              b[i] - wbase + (uint64_t)l > wlen) {
+            // (only a suffix array or LCP from a replay whose checks failed)
+            atomicExch(err, kDevRange);
+            ok = ok_b = false;
+          }
+          key[i] = ((uint64_t)w << (bl + bi)) | ((uint64_t)(lmax - l) << bi) | (uint64_t)(j + 1 - wbase);
+          a[i] -= wbase;
+          b[i] -= wbase;
+        }
+      }
+      okb[i] = __ballot_sync(0xffffffffu, ok);
+      ok_bb[i] = __ballot_sync(0xffffffffu, ok_b);
+      cnt += __popc(okb[i]) + __popc(ok_bb[i]);
+    }
+    uint32_t total;
+    const uint32_t ex = scan.run(cnt, OpSum(), &total);
+    if (threadIdx.x == 0 && total) s_base = atomicAdd(count, total);
+    __syncthreads();
+    uint32_t at = s_base + ex;
+    if (total) {
+#pragma unroll
+      for (int i = 0; i < kGenI; ++i) {
+        const uint32_t slot = at + __popc(okb[i] & lt) + __popc(ok_bb[i] & lt);
+        at += __popc(okb[i]) + __popc(ok_bb[i]);
+        if (!((okb[i] >> lane) & 1u)) continue;
+        const bool ok_b = (ok_bb[i] >> lane) & 1u;
+        if ((uint64_t)slot + (ok_b ? 1u : 0u) >= 2ull * (n - 1)) {
+          atomicExch(err, kDevRange);
+          continue;
+        }
+        const uint64_t ka = ks ? (key[i] << ks) | a[i] : key[i], kb = ks ? (key[i] << ks) | b[i] : key[i];
+        keys[slot] = ka;
+        if (ok_b) keys[slot + 1] = kb;
+        // the first digit: of the key when it holds the start, else of the value
+        atomicAdd(&sh[(ks ? (uint32_t)ka : a[i]) & hmask], 1u);
+        if (ok_b) atomicAdd(&sh[(ks ? (uint32_t)kb : b[i]) & hmask], 1u);
+        if (!ks) {  // the start is the value (otherwise it is the key's low digits)
+          vals[slot] = a[i];
+          if (ok_b) vals[slot + 1] = b[i];
+        }
       }
     }
-    uint64_t key = 0;
-    if (ok) {
-      // with several windows, the id and the start are relative to the
-      // window (its suffixes occupy a contiguous SA range starting at its
-      // offset), which keeps the key and value digits to the longest window
-      // (the pair's SA slots and suffixes lie in the same window: its id is
-      // read at slot k, next to the other threads' reads)
-      const uint32_t w = win_id(W, k), wbase = W.off_dev ? W.off_dev[w] : 0u;
-      const uint32_t wlen = (W.off_dev ? W.off_dev[w + 1] : n) - wbase;
-      if (a < wbase || b < wbase || a - wbase + (uint64_t)l > wlen || b - wbase + (uint64_t)l > wlen) {
-        // (only a suffix array or LCP from a replay whose checks failed)
-        atomicExch(err, kDevRange);
-        ok = ok_b = false;
-      }
-      const long long j = prev_less(T, k, l, err);
-      key = ((uint64_t)w << (bl + bi)) | ((uint64_t)(lmax - l) << bi) | (uint64_t)(j + 1 - wbase);
-      a -= wbase;
-      b -= wbase;
-    }
-    const uint32_t bal = __ballot_sync(0xffffffffu, ok), bal_b = __ballot_sync(0xffffffffu, ok_b);
-    if (bal == 0) continue;
-    const int leader = __ffs(bal) - 1;
-    uint32_t slot0 = 0;
-    if ((int)lane == leader) slot0 = atomicAdd(count, __popc(bal) + __popc(bal_b));
-    slot0 = __shfl_sync(0xffffffffu, slot0, leader);
-    if (ok) {
-      const uint32_t lt = lanemask_lt();
-      const uint32_t slot = slot0 + __popc(bal & lt) + __popc(bal_b & lt);
-      if (slot + (ok_b ? 1u : 0u) >= 2 * (n - 1)) {
-        atomicExch(err, kDevRange);
-        continue;
-      }
-      const uint64_t ka = ks ? (key << ks) | a : key, kb = ks ? (key << ks) | b : key;
-      keys[slot] = ka;
-      if (ok_b) keys[slot + 1] = kb;
-      // the first digit: of the key when it holds the start, else of the value
-      atomicAdd(&sh[(ks ? (uint32_t)ka : a) & hmask], 1u);
-      if (ok_b) atomicAdd(&sh[(ks ? (uint32_t)kb : b) & hmask], 1u);
-      if (!ks) {  // the start is the value (otherwise it is the key's low digits)
-        vals[slot] = a;
-        if (ok_b) vals[slot + 1] = b;
-      }
-    }
+    __syncthreads();  // s_base is read
   }
   __syncthreads();
-  for (uint32_t d = threadIdx.x; d <= hmask; d += blockDim.x)
+  for (uint32_t d = threadIdx.x; d <= hmask; d += kGenT)
     if (sh[d]) atomicAdd(&hist[d], sh[d]);
 }
 
@@ -564,17 +590,30 @@ __global__ void k_sel_out(const uint64_t *__restrict__ keys, const uint32_t *__r
 
 // First index of each window in a list sorted by window (the window of entry
 // k is the window of position pos[k]); out[count] = m.
+// One warp per window, 32 probes per step: a search over millions of entries
+// waits for memory five times instead of 25.
 __global__ void k_window_bounds(const uint32_t *__restrict__ pos, uint32_t m, Windows W, uint32_t n,
                                 uint32_t *__restrict__ out, const uint32_t *m_dev = nullptr) {
   if (m_dev) m = min(m, *m_dev);  // m: an upper bound
-  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w <= W.count; w += gridDim.x * blockDim.x) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w <= W.count; w += warps) {
+    auto before = [&](uint32_t k) {  // entry k belongs to an earlier window
+      const uint32_t p = pos[k];
+      return (p < n ? win_id(W, p) : W.count) < w;
+    };
     uint32_t lo = 0, hi = m;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi) >> 1;
-      const uint32_t p = pos[mid];
-      if ((p < n ? win_id(W, p) : W.count) < w) lo = mid + 1; else hi = mid;
+    while (hi - lo > 32) {
+      const uint32_t span = hi - lo;
+      const uint32_t q = lo + (uint32_t)((uint64_t)span * (lane + 1) / 33);
+      const uint32_t c = __popc(__ballot_sync(0xffffffffu, before(q)));
+      const uint32_t l2 = c ? lo + (uint32_t)((uint64_t)span * c / 33) + 1 : lo;
+      const uint32_t h2 = c < 32 ? lo + (uint32_t)((uint64_t)span * (c + 1) / 33) : hi;
+      lo = l2;
+      hi = h2;
     }
-    out[w] = lo;
+    lo += __popc(__ballot_sync(0xffffffffu, lo + lane < hi && before(lo + lane)));
+    if (lane == 0) out[w] = lo;
   }
 }
 
@@ -586,6 +625,21 @@ __global__ void k_relativize(uint32_t *__restrict__ start, uint32_t *__restrict_
     const uint32_t w = win_id(W, start[q]);
     if (trace) trace[q] -= trace_off[w];
     start[q] -= W.off_dev ? W.off_dev[w] : 0u;
+  }
+}
+
+// The caller's candidate arrays (null: not wanted), the first `k` candidates,
+// starts relative to their windows.
+__global__ void k_cand_out(const uint32_t *__restrict__ cl, const uint32_t *__restrict__ cid,
+                           const uint32_t *__restrict__ cs, const uint8_t *__restrict__ acc, uint64_t k, uint32_t n,
+                           Windows W, uint32_t *__restrict__ ol, uint32_t *__restrict__ oid, uint32_t *__restrict__ os,
+                           uint8_t *__restrict__ oa) {
+  for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < k; q += (uint64_t)gridDim.x * blockDim.x) {
+    if (ol) ol[q] = cl[q];
+    if (oid) oid[q] = cid[q];
+    // (a start past n: only a candidate of a replay whose checks failed)
+    if (os) os[q] = cs[q] - (W.off_dev && cs[q] < n ? W.off_dev[win_id(W, cs[q])] : 0u);
+    if (oa) oa[q] = acc[q];
   }
 }
 
@@ -806,7 +860,7 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int tb, const SuffixSta
   APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCandCount, 0, sizeof(uint32_t), s));
   {
     Launch lp_(c, kKCandGen, n, s);
-    k_cand_gen<<<g, 256, 0, s>>>(st.sa, lcp, n, min_len, T, bi, bl, lmax, ks, W, b.keys[0], b.vals[0],
+    k_cand_gen<<<std::max(1, std::min(ceil_div(n, kGenT * kGenI), c->num_sms * 8)), kGenT, 0, s>>>(st.sa, lcp, n, min_len, T, bi, bl, lmax, ks, W, b.keys[0], b.vals[0],
                                  misc + kMiscCandCount, c->ps.err, sort_first_hist(c),
                                  sp.shape >= 0 ? sp.bits : 8);
   }
@@ -846,7 +900,7 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int tb, const SuffixSta
   if (mu) {
     {
       Launch lp_(c, kKSlices, W.count + 1, s);
-      k_window_bounds<<<ceil_div(W.count + 1, 256), 256, 0, s>>>(cs, mu, W, n, cand_off, m_dev);
+      k_window_bounds<<<grid_for((uint64_t)(W.count + 1) * 32, 256, c->num_sms), 256, 0, s>>>(cs, mu, W, n, cand_off, m_dev);
     }
     APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscAccCount, 0, sizeof(uint32_t), s));
     APO_CUDA_TRY(cudaMemsetAsync(acc, 0, mu, s));
@@ -986,8 +1040,8 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int tb, const SuffixSta
     if (W.count > 1) {  // per-window offsets, then window-relative values
       {
         Launch lp_(c, kKSlices, W.count + 1, s);
-        k_window_bounds<<<ceil_div(W.count + 1, 256), 256, 0, s>>>(ss, K, W, n, sel_off);
-        k_window_bounds<<<ceil_div(W.count + 1, 256), 256, 0, s>>>(ts, Tn, W, n, trace_off);
+        k_window_bounds<<<grid_for((uint64_t)(W.count + 1) * 32, 256, c->num_sms), 256, 0, s>>>(ss, K, W, n, sel_off);
+        k_window_bounds<<<grid_for((uint64_t)(W.count + 1) * 32, 256, c->num_sms), 256, 0, s>>>(ts, Tn, W, n, trace_off);
       }
       {
         Launch lp_(c, kKSelOut, K, s);
@@ -996,17 +1050,16 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int tb, const SuffixSta
       }
     }
   }
-  if (W.count > 1 && m && out->cand_start) {
-    // window-relative candidate starts for the caller (greedy is done with them)
-    Launch lp_(c, kKSelOut, m, s);
-    k_relativize<<<grid_for(m, 256, c->num_sms), 256, 0, s>>>(cs, nullptr, m, W, trace_off);
-  }
-
   bool over = false;
-  APO_TRY(copy_out(out->cand_len, cl, m, out->cand_cap, &over, s));
-  APO_TRY(copy_out(out->cand_id, cid, m, out->cand_cap, &over, s));
-  APO_TRY(copy_out(out->cand_start, cs, m, out->cand_cap, &over, s));
-  APO_TRY(copy_out(out->cand_accepted, acc, m, out->cand_cap, &over, s));
+  if (out->cand_len || out->cand_id || out->cand_start || out->cand_accepted) {
+    over = m > out->cand_cap;
+    const uint64_t k = std::min<uint64_t>(m, out->cand_cap);
+    if (k) {
+      Launch lp_(c, kKSelOut, k, s);
+      k_cand_out<<<grid_for(k, 256, c->num_sms), 256, 0, s>>>(cl, cid, cs, acc, k, n, W, out->cand_len, out->cand_id,
+                                                              out->cand_start, out->cand_accepted);
+    }
+  }
   APO_TRY(copy_out(out->sel_start, ss, K, out->sel_cap, &over, s));
   APO_TRY(copy_out(out->sel_len, sl, K, out->sel_cap, &over, s));
   APO_TRY(copy_out(out->sel_trace, sq, K, out->sel_cap, &over, s));

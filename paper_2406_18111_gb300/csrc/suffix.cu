@@ -69,24 +69,46 @@ __global__ void k_init_keys(const void *__restrict__ tokens, int tb, uint32_t n,
   }
 }
 
-// out[0] |= every token, out[1] = max(out[1], every token).
-__global__ void k_token_or(const void *__restrict__ tokens, int tb, uint32_t n, unsigned long long *out) {
-  uint64_t acc = 0, mx = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint64_t k = tb == 4 ? (uint64_t) static_cast<const uint32_t *>(tokens)[i]
-                               : static_cast<const uint64_t *>(tokens)[i];
-    acc |= k;
-    mx = k > mx ? k : mx;
+// out[0] |= every token, out[1] = max(out[1], every token).  Eight loads in
+// flight per thread: a stream over the tokens.
+constexpr int kOrT = 256, kOrI = 8;
+template <class T>
+__global__ void __launch_bounds__(kOrT) k_token_or(const T *__restrict__ tokens, uint32_t n,
+                                                   unsigned long long *out) {
+  T acc = 0, mx = 0;
+  const uint64_t stride = (uint64_t)gridDim.x * kOrT * kOrI;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * kOrT * kOrI + threadIdx.x; i0 < n; i0 += stride) {
+    T v[kOrI];
+#pragma unroll
+    for (int j = 0; j < kOrI; ++j) v[j] = i0 + j * kOrT < n ? tokens[i0 + j * kOrT] : (T)0;
+#pragma unroll
+    for (int j = 0; j < kOrI; ++j) {
+      acc |= v[j];
+      mx = v[j] > mx ? v[j] : mx;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     acc |= __shfl_xor_sync(0xffffffffu, acc, o);
-    const uint64_t m2 = __shfl_xor_sync(0xffffffffu, mx, o);
+    const T m2 = __shfl_xor_sync(0xffffffffu, mx, o);
     mx = m2 > mx ? m2 : mx;
   }
-  if ((threadIdx.x & 31) == 0 && acc) {
-    atomicOr(out, (unsigned long long)acc);
-    atomicMax(out + 1, (unsigned long long)mx);
+  __shared__ T s_or[kOrT / 32], s_mx[kOrT / 32];
+  if ((threadIdx.x & 31) == 0) {
+    s_or[threadIdx.x >> 5] = acc;
+    s_mx[threadIdx.x >> 5] = mx;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < kOrT / 32; ++w) {
+      acc |= s_or[w];
+      mx = s_mx[w] > mx ? s_mx[w] : mx;
+    }
+    if (acc) {
+      atomicOr(out, (unsigned long long)acc);
+      atomicMax(out + 1, (unsigned long long)mx);
+    }
   }
 }
 
@@ -281,28 +303,33 @@ __device__ __forceinline__ uint64_t token_at(const void *tokens, int tb, uint32_
 
 // Inserts every token (a token equal to the empty marker gets the last code
 // by itself, see k_code_map); counts distinct tokens and gives up (flag)
-// past `limit` of them.
+// past `limit` of them.  A warp adds its new tokens to the count at once:
+// with one addition per new token, 2^22 of them (a window of random tokens,
+// where the dictionary is given up) queued on one address for 0.8 ms.
 __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t n, uint64_t *keys, uint64_t mask,
                               uint32_t limit, uint32_t *distinct, uint32_t *over) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (*(volatile uint32_t *)over) return;
-    const uint64_t t = token_at(tokens, tb, i);
-    if (t == kDictEmpty) continue;
-    uint64_t slot = dmix(t) & mask;
-    for (uint64_t probe = 0; probe <= mask; ++probe) {
-      uint64_t cur = keys[slot];
-      if (cur == t) break;
-      if (cur == kDictEmpty) {
-        cur = atomicCAS((unsigned long long *)&keys[slot], (unsigned long long)kDictEmpty,
-                        (unsigned long long)t);
-        if (cur == kDictEmpty) {
-          if (atomicAdd(distinct, 1u) >= limit) atomicExch(over, 1u);
-          break;
-        }
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
+    if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) return;
+    const uint64_t i = i0 + lane;
+    bool fresh = false;
+    const uint64_t t = i < n ? token_at(tokens, tb, (uint32_t)i) : kDictEmpty;
+    if (t != kDictEmpty) {
+      uint64_t slot = dmix(t) & mask;
+      for (uint64_t probe = 0; probe <= mask; ++probe) {
+        uint64_t cur = keys[slot];
         if (cur == t) break;
+        if (cur == kDictEmpty) {
+          cur = atomicCAS((unsigned long long *)&keys[slot], (unsigned long long)kDictEmpty, (unsigned long long)t);
+          fresh = cur == kDictEmpty;
+          if (fresh || cur == t) break;
+        }
+        slot = (slot + 1) & mask;
       }
-      slot = (slot + 1) & mask;
     }
+    const uint32_t c = __popc(__ballot_sync(0xffffffffu, fresh));
+    if (lane == 0 && c && atomicAdd(distinct, c) + c > limit) atomicExch(over, 1u);
   }
 }
 
@@ -1272,8 +1299,12 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
   APO_CUDA_TRY(cudaMemsetAsync(kor, 0, 2 * sizeof(uint64_t), s));
   {
     Launch lp_(c, kKKeyOr, n, s);
-    k_token_or<<<std::min(1024, ceil_div(n, 256 * 8)), 256, 0, s>>>(tokens, tb, n,
-                                                                     reinterpret_cast<unsigned long long *>(kor));
+    const int ob = std::max(1, std::min(c->num_sms * 8, ceil_div(n, kOrT * kOrI)));
+    unsigned long long *ko = reinterpret_cast<unsigned long long *>(kor);
+    if (tb == 4)
+      k_token_or<<<ob, kOrT, 0, s>>>(static_cast<const uint32_t *>(tokens), n, ko);
+    else
+      k_token_or<<<ob, kOrT, 0, s>>>(static_cast<const uint64_t *>(tokens), n, ko);
   }
   DictCodes dict;
   const bool dict_early = tb == 8 && n >= 4096;
