@@ -119,22 +119,46 @@ struct Dict {
   uint64_t mask;
 };
 
+// Four tokens per thread, whose first slots' reads are under way together.
+// Lanes that find the same slot empty leave the insertion to the first of
+// them: the tokens of a task stream are few, and the first reads of the whole
+// chip see them missing.
+constexpr int kDictI = 4;
 template <class T>
 __global__ void k_dict_insert(const T *__restrict__ tok, uint64_t m, Dict d) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t t = (uint64_t)tok[i];
-    if (t == kEmpty) continue;  // mapped to a reserved symbol instead
-    uint64_t slot = mix64(t) & d.mask;
-    for (uint64_t probe = 0; probe <= d.mask; ++probe) {
-      uint64_t cur = d.keys[slot];
-      if (cur == t) break;
-      if (cur == kEmpty) {
-        cur = atomicCAS((unsigned long long *)&d.keys[slot], (unsigned long long)kEmpty,
-                        (unsigned long long)t);
-        if (cur == kEmpty || cur == t) break;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kDictI;
+  const uint32_t lt = lanemask_lt();
+  for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kDictI; b0 < m; b0 += stride) {
+    uint64_t t[kDictI], cur[kDictI];
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) {  // (all-ones: mapped to a reserved symbol instead)
+      const uint64_t i = b0 + (uint64_t)u * blockDim.x + threadIdx.x;
+      t[u] = i < m ? (uint64_t)tok[i] : kEmpty;
+    }
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) cur[u] = t[u] != kEmpty ? d.keys[mix64(t[u]) & d.mask] : kEmpty;
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) {
+      uint64_t slot = mix64(t[u]) & d.mask;
+      const bool need = t[u] != kEmpty && cur[u] == kEmpty;
+      if (__any_sync(0xffffffffu, need)) {
+        const uint32_t peers = __match_any_sync(0xffffffffu, need ? (uint32_t)slot : ~0u);
+        if (need && (peers & lt) == 0)
+          cur[u] = atomicCAS((unsigned long long *)&d.keys[slot], (unsigned long long)kEmpty, (unsigned long long)t[u]);
+        const uint64_t first = __shfl_sync(0xffffffffu, cur[u], __ffs(peers) - 1);
+        const uint64_t by = __shfl_sync(0xffffffffu, t[u], __ffs(peers) - 1);
+        if (need) cur[u] = first == kEmpty ? by : first;  // what the slot holds now
       }
-      slot = (slot + 1) & d.mask;
+      if (t[u] == kEmpty || cur[u] == t[u]) continue;
+      for (uint64_t probe = 0; probe <= d.mask; ++probe) {
+        slot = (slot + 1) & d.mask;
+        uint64_t c = d.keys[slot];
+        if (c == t[u]) break;
+        if (c == kEmpty) {
+          c = atomicCAS((unsigned long long *)&d.keys[slot], (unsigned long long)kEmpty, (unsigned long long)t[u]);
+          if (c == kEmpty || c == t[u]) break;
+        }
+      }
     }
   }
 }
@@ -154,9 +178,24 @@ __device__ __forceinline__ uint32_t dict_symbol(const Dict &d, T tok) {
 
 template <class T>
 __global__ void k_dict_map(const T *__restrict__ tok, uint64_t m, Dict d, uint32_t *__restrict__ sym) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    sym[i] = dict_symbol(d, tok[i]);
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kDictI;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * kDictI + threadIdx.x; i0 < m; i0 += stride) {
+    uint64_t t[kDictI], cur[kDictI];
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) {
+      const uint64_t i = i0 + (uint64_t)u * blockDim.x;
+      t[u] = i < m ? (uint64_t)tok[i] : kEmpty;
+    }
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) cur[u] = d.keys[mix64(t[u]) & d.mask];
+#pragma unroll
+    for (int u = 0; u < kDictI; ++u) {
+      const uint64_t i = i0 + (uint64_t)u * blockDim.x;
+      if (i >= m) continue;
+      const uint64_t slot = mix64(t[u]) & d.mask;
+      sym[i] = t[u] != kEmpty && cur[u] == t[u] ? (uint32_t)slot : dict_symbol(d, (T)t[u]);
+    }
+  }
 }
 
 // max length, max end and total length of slice-form patterns; flags empty ones
@@ -455,7 +494,8 @@ struct SrcReachSrc {
 
 // ---------------------------------------------------------------- nodes and links
 struct NodeArgs {
-  const uint32_t *tstart, *plen, *tsym;
+  const uint32_t *tstart, *plen, *tsym, *tpid;
+  uint32_t N;              // positions of T
   const uint32_t *jpos, *sp, *sr;  // sorted starts: pattern sp[j] at SA index sr[j]
   const uint32_t *rank, *left, *reach;
   Sparse S;  // minima over slcp
@@ -496,8 +536,11 @@ __device__ __forceinline__ uint32_t node_of(const NodeArgs &a, uint32_t j, uint3
   return a.tstart[a.sp[rep_of(a.S, j, d)]] + d - 1;
 }
 
-// One warp per pattern, one lane per depth d = 1 .. len + 1 (len + 1 is the
-// separator after the pattern).  A depth-d prefix that is its own node gets
+// One thread per position of T: depth d = 1 .. len + 1 of its pattern (len + 1
+// is the separator after it).  A node costs some 40 dependent reads, so what
+// bounds the kernel is how many are under way; with a warp per pattern the
+// longest patterns set the pace (790 us for 10,000 patterns of up to 2,000
+// symbols).  A depth-d prefix that is its own node gets
 // its failure link, and the branch edge into it when it hangs off another
 // pattern's node; the pattern's end node counts one more pattern end.  With
 // `pref`, every node also gets its preferred child: the one that the most
@@ -506,69 +549,64 @@ __device__ __forceinline__ uint32_t node_of(const NodeArgs &a, uint32_t j, uint3
 // children are wanted by the halo pass only, which is when kPref is set.
 template <bool kPref>
 __global__ void k_ac_nodes(NodeArgs a) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < a.P; i += warps) {
-    const uint32_t S = a.tstart[i], len = a.plen[i], j = a.jpos[i];
-    const uint32_t sl = a.S.lev[0][j];
-    for (uint32_t d = lane + 1; d <= len + 1; d += 32) {
-      const uint32_t v = S + d - 1;
-      uint32_t f = a.root;
-      if (d <= len && d > sl) {
-        const uint32_t e = S + d;
-        if (d >= 2 && a.reach[e - 1] >= e) {
-          uint32_t lo = S + 1, hi = e - 1;  // first q in (S, e) with reach >= e
-          while (lo < hi) {
-            const uint32_t mid = lo + ((hi - lo) >> 1);
-            if (a.reach[mid] >= e) hi = mid;
-            else lo = mid + 1;
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < a.N; v += gridDim.x * blockDim.x) {
+    const uint32_t i = a.tpid[v], S = a.tstart[i], len = a.plen[i], j = a.jpos[i];
+    const uint32_t sl = a.S.lev[0][j], d = v - S + 1;
+    uint32_t f = a.root;
+    if (d <= len && d > sl) {
+      const uint32_t e = S + d;
+      if (d >= 2 && a.reach[e - 1] >= e) {
+        uint32_t lo = S + 1, hi = e - 1;  // first q in (S, e) with reach >= e
+        while (lo < hi) {
+          const uint32_t mid = lo + ((hi - lo) >> 1);
+          if (a.reach[mid] >= e) hi = mid;
+          else lo = mid + 1;
+        }
+        const uint32_t fd = e - lo;
+        if (a.src) {
+          // the string's LCP interval in the source; the first pattern in
+          // sorted order whose key is not below (left end, fd) starts with it
+          const uint32_t r = a.src_rank[a.pstart[i] + (lo - S)];
+          const uint64_t key = ((uint64_t)(prev_less(a.T, r, fd, a.err) + 1) << a.lenbits) | fd;
+          uint32_t jl = 0, jh = a.P;
+          while (jl < jh) {
+            const uint32_t mid = (jl + jh) >> 1;
+            if (a.skey[mid] < key) jl = mid + 1;
+            else jh = mid;
           }
-          const uint32_t fd = e - lo;
-          if (a.src) {
-            // the string's LCP interval in the source; the first pattern in
-            // sorted order whose key is not below (left end, fd) starts with it
-            const uint32_t r = a.src_rank[a.pstart[i] + (lo - S)];
-            const uint64_t key = ((uint64_t)(prev_less(a.T, r, fd, a.err) + 1) << a.lenbits) | fd;
-            uint32_t jl = 0, jh = a.P;
-            while (jl < jh) {
-              const uint32_t mid = (jl + jh) >> 1;
-              if (a.skey[mid] < key) jl = mid + 1;
-              else jh = mid;
-            }
-            if (jl >= a.P) atomicExch(a.err, kDevRange);
-            else f = a.tstart[a.sp[jl]] + fd - 1;
+          if (jl >= a.P) atomicExch(a.err, kDevRange);
+          else f = a.tstart[a.sp[jl]] + fd - 1;
+        } else {
+          const uint32_t k = a.rank[lo];
+          uint32_t cnt = 0, hi2 = a.P;  // starts before SA index k
+          while (cnt < hi2) {
+            const uint32_t mid = (cnt + hi2) >> 1;
+            if (a.sr[mid] < k) cnt = mid + 1;
+            else hi2 = mid;
+          }
+          const uint32_t jj = (a.left[k] >= fd) ? cnt - 1 : cnt;
+          if (jj >= a.P) {
+            atomicExch(a.err, kDevRange);
           } else {
-            const uint32_t k = a.rank[lo];
-            uint32_t cnt = 0, hi2 = a.P;  // starts before SA index k
-            while (cnt < hi2) {
-              const uint32_t mid = (cnt + hi2) >> 1;
-              if (a.sr[mid] < k) cnt = mid + 1;
-              else hi2 = mid;
-            }
-            const uint32_t jj = (a.left[k] >= fd) ? cnt - 1 : cnt;
-            if (jj >= a.P) {
-              atomicExch(a.err, kDevRange);
-            } else {
-              f = node_of(a, jj, fd);
-            }
+            f = node_of(a, jj, fd);
           }
         }
-        if (d == sl + 1) {
-          const uint32_t parent = d == 1 ? a.root : node_of(a, j, d - 1);
-          table_insert(a.g, parent, a.tsym[v], v, a.err);
-          a.has_branch[parent] = 1;
-          if (kPref && d > 1)  // v as a child of parent, weighed by the patterns through it
-            atomicMax(&a.pref[parent], ((unsigned long long)(block_end(a.S, j, d, a.P) - j) << 32) | v);
-        }
-        if (kPref && d < len)  // v's own next position as its child
-          atomicMax(&a.pref[v], ((unsigned long long)(block_end(a.S, j, d + 1, a.P) - j) << 32) | (v + 1));
       }
-      a.fail[v] = f;
-      if (d == len) {
-        const uint32_t en = node_of(a, j, len);
-        a.end_node[i] = en;
-        atomicAdd(&a.own[en], 1u);
+      if (d == sl + 1) {
+        const uint32_t parent = d == 1 ? a.root : node_of(a, j, d - 1);
+        table_insert(a.g, parent, a.tsym[v], v, a.err);
+        a.has_branch[parent] = 1;
+        if (kPref && d > 1)  // v as a child of parent, weighed by the patterns through it
+          atomicMax(&a.pref[parent], ((unsigned long long)(block_end(a.S, j, d, a.P) - j) << 32) | v);
       }
+      if (kPref && d < len)  // v's own next position as its child
+        atomicMax(&a.pref[v], ((unsigned long long)(block_end(a.S, j, d + 1, a.P) - j) << 32) | (v + 1));
+    }
+    a.fail[v] = f;
+    if (d == len) {
+      const uint32_t en = node_of(a, j, len);
+      a.end_node[i] = en;
+      atomicAdd(&a.own[en], 1u);
     }
   }
 }
@@ -717,52 +755,6 @@ __global__ void k_flat_chains(const uint4 *__restrict__ rec, uint32_t R, const u
       for (uint32_t k = lane; k < q.y; k += 32) flat[o + k] = evals[q.x + k];
       o += q.y;
       cur = q.z;
-    }
-  }
-}
-
-// Pass B over flattened chains: one warp per 32 positions; lane j fetches
-// position x0+j's chain; short chains are copied by their own lane, long ones
-// by the whole warp in position order (contiguous reads and writes).
-constexpr uint32_t kFillOwn = 4;
-__global__ void k_ac_fill_flat(const uint32_t *__restrict__ state, uint32_t n, const uint32_t *__restrict__ off,
-                               const uint32_t *__restrict__ firstrec, const uint32_t *__restrict__ rtot,
-                               const uint32_t *__restrict__ flat_off, const uint32_t *__restrict__ flat,
-                               uint32_t *mend, uint32_t *mid, uint64_t cap) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint64_t x0 = (uint64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; x0 < n;
-       x0 += (uint64_t)warps * 32) {
-    const uint64_t x = x0 + lane;
-    uint32_t cnt = 0, src = 0, dst = 0;
-    if (x < n) {
-      const uint32_t r = firstrec[state[x]];
-      if (r != kNil) {
-        cnt = rtot[r];
-        src = flat_off[r];
-        dst = off[x];
-      }
-    }
-    if (cnt <= kFillOwn) {  // short chains: each lane copies its own
-      for (uint32_t k = 0; k < cnt; ++k) {
-        if (dst + (uint64_t)k < cap) {
-          mend[dst + k] = (uint32_t)x;
-          mid[dst + k] = flat[src + k];
-        }
-      }
-    }
-    for (uint32_t busy = __ballot_sync(0xffffffffu, cnt > kFillOwn); busy; busy &= busy - 1) {
-      const int j = __ffs(busy) - 1;
-      const uint32_t c = __shfl_sync(0xffffffffu, cnt, j);
-      const uint32_t sj = __shfl_sync(0xffffffffu, src, j);
-      const uint64_t dj = __shfl_sync(0xffffffffu, dst, j);
-      const uint32_t xj = (uint32_t)(x0 + j);
-      for (uint32_t k = lane; k < c; k += 32) {
-        if (dj + k < cap) {
-          mend[dj + k] = xj;
-          mid[dj + k] = flat[sj + k];
-        }
-      }
     }
   }
 }
@@ -1115,7 +1107,86 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
     if (seg + i * 32 < n) off[seg + i * 32] = r + inc[i] - v[i];
 }
 
-// Pass B: the matches of position x, down the output chain from its state
+// Pass B over flattened chains, offsets and matches in one pass: a tile counts
+// its positions' matches, a look-back sum gives the first output place, and
+// each row of 32 positions is copied from the flattened chains: short ones by
+// their own lane, long ones by the whole warp in position order (contiguous
+// reads and writes).  Offsets written and read back cost two more passes over
+// the positions (2^26 of them: 315 us for the offsets, 341 for the copy).
+// I: rows per warp; fewer on short streams, for more tiles.
+constexpr uint32_t kFillOwn = 4;
+constexpr int kFT = 512;
+template <int I>
+__global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__ state, uint32_t n,
+                                                    const uint32_t *__restrict__ firstrec,
+                                                    const uint32_t *__restrict__ rtot,
+                                                    const uint32_t *__restrict__ flat_off,
+                                                    const uint32_t *__restrict__ flat, uint32_t *__restrict__ mend,
+                                                    uint32_t *__restrict__ mid, uint64_t cap, uint32_t *sum_out,
+                                                    uint64_t *status, uint32_t *tile_ctr, uint32_t epoch,
+                                                    uint32_t *err) {
+  __shared__ uint32_t s_tile, s_pre, s_scan[2 * kFT / 32];
+  WarpScan<kFT / 32> scan{s_scan, 0};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
+  __syncthreads();
+  const uint32_t t = s_tile;
+  const uint64_t base = (uint64_t)t * (kFT * I);
+  const uint64_t seg = base + (uint64_t)warp * (I * 32) + lane;
+  uint32_t rec[I], cnt[I], sum = 0;
+#pragma unroll
+  for (int i = 0; i < I; ++i) rec[i] = seg + i * 32 < n ? state[seg + i * 32] : kNil;
+#pragma unroll
+  for (int i = 0; i < I; ++i) rec[i] = rec[i] != kNil ? firstrec[rec[i]] : kNil;
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    cnt[i] = rec[i] != kNil ? rtot[rec[i]] : 0u;
+    sum += cnt[i];
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  uint32_t tot;
+  const uint32_t ex = scan.run(sum, OpSum(), &tot);
+  if (warp == 0) {
+    const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
+    if (lane == 0) {
+      s_pre = pre;
+      if (base + kFT * I >= n) *sum_out = pre + tot;
+    }
+  }
+  __syncthreads();
+  uint32_t at = s_pre + ex;
+  if (sum == 0) return;  // (the whole warp)
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const uint32_t inc = warp_inclusive(cnt[i], OpSum());
+    const uint32_t dst = at + inc - cnt[i], c0 = cnt[i];
+    at += __shfl_sync(0xffffffffu, inc, 31);
+    const uint32_t src = c0 ? flat_off[rec[i]] : 0u;
+    const uint32_t x = (uint32_t)(seg + i * 32);
+    if (c0 <= kFillOwn) {  // short chains: each lane copies its own
+      for (uint32_t k = 0; k < c0; ++k) {
+        if (dst + (uint64_t)k < cap) {
+          mend[dst + k] = x;
+          mid[dst + k] = flat[src + k];
+        }
+      }
+    }
+    for (uint32_t busy = __ballot_sync(0xffffffffu, c0 > kFillOwn); busy; busy &= busy - 1) {
+      const int j = __ffs(busy) - 1;
+      const uint32_t c = __shfl_sync(0xffffffffu, c0, j), sj = __shfl_sync(0xffffffffu, src, j);
+      const uint64_t dj = __shfl_sync(0xffffffffu, dst, j);
+      const uint32_t xj = __shfl_sync(0xffffffffu, x, j);
+      for (uint32_t k = lane; k < c; k += 32) {
+        if (dj + k < cap) {
+          mend[dj + k] = xj;
+          mid[dj + k] = flat[sj + k];
+        }
+      }
+    }
+  }
+}
+
+// Pass B for chains too long to flatten: the matches of position x, down the output chain from its state
 // (deepest first), ids ascending within a node.  The chain is walked over
 // the compact output records (one 16-byte load per node that ends patterns).
 __global__ void k_ac_fill(const uint32_t *__restrict__ state, uint32_t n, const uint32_t *__restrict__ off,
@@ -1345,10 +1416,10 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   {
     Launch lp_(c, kKDictInsert, extent, s);
     if (tb == 4)
-      k_dict_insert<<<grid_for(extent, 256, sms), 256, 0, s>>>(static_cast<const uint32_t *>(pp->tokens),
+      k_dict_insert<<<grid_for((extent + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint32_t *>(pp->tokens),
                                                                 extent, d);
     else
-      k_dict_insert<<<grid_for(extent, 256, sms), 256, 0, s>>>(static_cast<const uint64_t *>(pp->tokens),
+      k_dict_insert<<<grid_for((extent + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint64_t *>(pp->tokens),
                                                                 extent, d);
   }
   {
@@ -1364,9 +1435,9 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   if (n) {
     Launch lp_(c, kKDictMap, n, s);
     if (tb == 4)
-      k_dict_map<<<grid_for(n, 256, sms), 256, 0, s>>>(static_cast<const uint32_t *>(stream), n, d, ssym);
+      k_dict_map<<<grid_for((n + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint32_t *>(stream), n, d, ssym);
     else
-      k_dict_map<<<grid_for(n, 256, sms), 256, 0, s>>>(static_cast<const uint64_t *>(stream), n, d, ssym);
+      k_dict_map<<<grid_for((n + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint64_t *>(stream), n, d, ssym);
   }
   APO_CUDA_TRY(cudaGetLastError());
 
@@ -1484,6 +1555,8 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     a.tstart = tstart;
     a.plen = plen;
     a.tsym = tsym;
+    a.tpid = tpid;
+    a.N = N;
     a.jpos = jpos;
     a.sp = sp;
     a.sr = sr;
@@ -1508,9 +1581,9 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     a.lenbits = lenbits;
     Launch lp_(c, kKAcNodes, N, s);
     if (pref)
-      k_ac_nodes<true><<<std::max(1, std::min(ceil_div(P, 8), sms * 16)), 256, 0, s>>>(a);
+      k_ac_nodes<true><<<grid_for(N, 256, sms), 256, 0, s>>>(a);
     else
-      k_ac_nodes<false><<<std::max(1, std::min(ceil_div(P, 8), sms * 16)), 256, 0, s>>>(a);
+      k_ac_nodes<false><<<grid_for(N, 256, sms), 256, 0, s>>>(a);
   }
   // pattern ids grouped by end node
   {
@@ -1553,12 +1626,16 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     }
     APO_TRY(seg_scan<false>(c, SrcU32{rtot}, DstExclusive{rtot, flat_off, misc + kMiscFlatTotal, P}, P, OpSum(),
                             0u, s));
+    // read while the states are computed
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 1, misc + kMiscTraceCount, 4, cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscFlatTotal, 4, cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaEventRecord(c->round_ev[0], s));
   }
 
   // pass A: the state of every stream position (pass shape chosen above)
   Automaton A{tsym, has_branch, g, skip, root, {skip}, (uint32_t)(maxlen / 32 + 2), {}};
   uint32_t *state = c->arena.take_n<uint32_t>(n);
-  uint32_t *off = c->arena.take_n<uint32_t>(n);
+  uint32_t *off = c->arena.take_n<uint32_t>(n);  // (offsets: only without flattened chains)
   if (!state || !off) return APO_ENOMEM;
   if (halo) {
     // lifting tables of the skip links and of the preferred children
@@ -1601,11 +1678,41 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     APO_CUDA_TRY(cudaStreamSynchronize(s));
     if (c->host_pinned[0] == 0) break;
   }
-  // output offsets and total
-  const int tiles = ceil_div(n, kSTile);
+  // Flatten each output record's chain once (the sum over records of their
+  // chain lengths is usually far below the match count), then copy chains per
+  // position.  Very long flattened chains fall back to walking.
+  uint32_t R = 0;
+  uint64_t flat_total = ~0ull;
+  if (flat_ok) {
+    APO_CUDA_TRY(cudaEventSynchronize(c->round_ev[0]));
+    R = c->host_pinned[1];
+    if (R) flat_total = c->host_pinned[2];
+  }
+  const uint64_t flat_bytes = std::max<uint64_t>(flat_total, 1) * 4;
+  const bool flat = flat_total <= kMaxFlat;
+  // (with a caller workspace too small a side buffer is an error only once
+  // there is a match to write)
+  const bool fused = flat && !(c->ext && flat_bytes > c->side_bytes);
+  auto flatten = [&]() -> int {
+    APO_TRY(ensure_side(c, flat_bytes, s));
+    Launch lp_(c, kKAcFill, flat_total, s);
+    k_flat_chains<<<std::max(1, std::min(ceil_div(R, 8), sms * 16)), 256, 0, s>>>(rec, R, flat_off, ev,
+                                                                                  static_cast<uint32_t *>(c->side));
+    APO_CUDA_TRY(cudaGetLastError());
+    return APO_OK;
+  };
+  if (fused) APO_TRY(flatten());
+  // matches (or their offsets) and their total
+  const bool wide = n >= (1ull << 22);
+  const int tiles = fused ? ceil_div(n, kFT * (wide ? 8 : 2)) : ceil_div(n, kSTile);
   APO_TRY(ensure_lookback(c, tiles));
   APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
-  {
+  if (fused) {
+    Launch lp_(c, kKAcFill, n, s);
+    (wide ? k_match_fill<8> : k_match_fill<2>)<<<tiles, kFT, 0, s>>>(
+        state, (uint32_t)n, firstrec, rtot, flat_off, static_cast<const uint32_t *>(c->side), match_end, match_id, cap,
+        misc + kMiscCompactCount, c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c), c->ps.err);
+  } else {
     Launch lp_(c, kKMatchOffsets, n, s);
     k_match_offsets<<<tiles, kST, 0, s>>>(state, mtotal, (uint32_t)n, off, misc + kMiscCompactCount,
                                           c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c),
@@ -1613,9 +1720,6 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   }
   APO_CUDA_TRY(cudaGetLastError());
   APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned, misc + kMiscCompactCount, 4, cudaMemcpyDeviceToHost, s));
-  APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 1, misc + kMiscTraceCount, 4, cudaMemcpyDeviceToHost, s));
-  if (flat_ok)
-    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscFlatTotal, 4, cudaMemcpyDeviceToHost, s));
   APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + kPinnedErr, c->ps.err, sizeof(uint32_t),
                                cudaMemcpyDeviceToHost, s));
   APO_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1626,30 +1730,12 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     set_error("match_candidates: more matches than cap (count written)");
     return APO_ECAPACITY;
   }
-  if (total_m) {
-    // flatten each output record's chain once (sum over records of their
-    // chain lengths, usually far below the match count), then copy chains
-    // per position; very long flattened chains fall back to walking
-    const uint32_t R = c->host_pinned[1];
-    const uint64_t flat_total = flat_ok && R ? c->host_pinned[2] : ~0ull;
-    uint32_t *flat = nullptr;
-    if (flat_total <= kMaxFlat) {
-      APO_TRY(ensure_side(c, std::max<uint64_t>(flat_total, 1) * 4, s));
-      flat = static_cast<uint32_t *>(c->side);
-    }
-    if (flat) {
-      {
-        Launch lp_(c, kKAcFill, flat_total, s);
-        k_flat_chains<<<std::max(1, std::min(ceil_div(R, 8), sms * 16)), 256, 0, s>>>(rec, R, flat_off, ev, flat);
-      }
-      Launch lp_(c, kKAcFill, n, s);
-      k_ac_fill_flat<<<std::max(1, std::min(ceil_div(n, 256), sms * 32)), 256, 0, s>>>(
-          state, (uint32_t)n, off, firstrec, rtot, flat_off, flat, match_end, match_id, cap);
-    } else {
-      Launch lp_(c, kKAcFill, n, s);
-      k_ac_fill<<<grid_for(n, 256, sms), 256, 0, s>>>(state, (uint32_t)n, off, firstrec, rec, ev, match_end,
-                                                      match_id, cap);
-    }
+  if (fused || !total_m) return APO_OK;  // synchronised above
+  if (flat) APO_TRY(flatten());  // (a caller workspace: no room, an error)
+  {
+    Launch lp_(c, kKAcFill, n, s);
+    k_ac_fill<<<grid_for(n, 256, sms), 256, 0, s>>>(state, (uint32_t)n, off, firstrec, rec, ev, match_end,
+                                                    match_id, cap);
   }
   APO_CUDA_TRY(cudaGetLastError());
   return check_device_error(c, s);  // synchronises

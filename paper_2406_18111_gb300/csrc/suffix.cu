@@ -308,27 +308,48 @@ __device__ __forceinline__ uint64_t token_at(const void *tokens, int tb, uint32_
 // where the dictionary is given up) queued on one address for 0.8 ms.
 __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t n, uint64_t *keys, uint64_t mask,
                               uint32_t limit, uint32_t *distinct, uint32_t *over) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
+  constexpr int kI = 4;  // tokens per thread: their first slots' reads are under way together
+  const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kI;
+  for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kI; b0 < n; b0 += stride) {
     if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) return;
-    const uint64_t i = i0 + lane;
-    bool fresh = false;
-    const uint64_t t = i < n ? token_at(tokens, tb, (uint32_t)i) : kDictEmpty;
-    if (t != kDictEmpty) {
-      uint64_t slot = dmix(t) & mask;
-      for (uint64_t probe = 0; probe <= mask; ++probe) {
-        uint64_t cur = keys[slot];
-        if (cur == t) break;
-        if (cur == kDictEmpty) {
-          cur = atomicCAS((unsigned long long *)&keys[slot], (unsigned long long)kDictEmpty, (unsigned long long)t);
-          fresh = cur == kDictEmpty;
-          if (fresh || cur == t) break;
+    uint64_t t[kI], cur[kI];
+    uint32_t fresh = 0;
+#pragma unroll
+    for (int u = 0; u < kI; ++u) {
+      const uint64_t i = b0 + (uint64_t)u * blockDim.x + threadIdx.x;
+      t[u] = i < n ? token_at(tokens, tb, (uint32_t)i) : kDictEmpty;
+    }
+#pragma unroll
+    for (int u = 0; u < kI; ++u) cur[u] = t[u] != kDictEmpty ? keys[dmix(t[u]) & mask] : kDictEmpty;
+#pragma unroll
+    for (int u = 0; u < kI; ++u) {
+      uint64_t slot = dmix(t[u]) & mask;
+      const bool need = t[u] != kDictEmpty && cur[u] == kDictEmpty;
+      if (__any_sync(0xffffffffu, need)) {
+        // lanes that find the same slot empty leave the insertion to the first
+        const uint32_t peers = __match_any_sync(0xffffffffu, need ? (uint32_t)slot : ~0u);
+        if (need && (peers & lt) == 0) {
+          cur[u] = atomicCAS((unsigned long long *)&keys[slot], (unsigned long long)kDictEmpty, (unsigned long long)t[u]);
+          if (cur[u] == kDictEmpty) ++fresh;
         }
+        const uint64_t first = __shfl_sync(0xffffffffu, cur[u], __ffs(peers) - 1);
+        const uint64_t by = __shfl_sync(0xffffffffu, t[u], __ffs(peers) - 1);
+        if (need) cur[u] = first == kDictEmpty ? by : first;  // what the slot holds now
+      }
+      if (t[u] == kDictEmpty || cur[u] == t[u]) continue;
+      for (uint64_t probe = 0; probe <= mask; ++probe) {
         slot = (slot + 1) & mask;
+        uint64_t c = keys[slot];
+        if (c == t[u]) break;
+        if (c == kDictEmpty) {
+          c = atomicCAS((unsigned long long *)&keys[slot], (unsigned long long)kDictEmpty, (unsigned long long)t[u]);
+          if (c == kDictEmpty) ++fresh;
+          if (c == kDictEmpty || c == t[u]) break;
+        }
       }
     }
-    const uint32_t c = __popc(__ballot_sync(0xffffffffu, fresh));
+    const uint32_t c = __reduce_add_sync(0xffffffffu, fresh);
     if (lane == 0 && c && atomicAdd(distinct, c) + c > limit) atomicExch(over, 1u);
   }
 }
@@ -1190,7 +1211,7 @@ int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCod
   APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDict, 0, 2 * sizeof(uint32_t), s));
   {
     Launch lp_(c, kKSaDict, n, s);
-    k_dict_tokens<<<grid_for(n, 256, c->num_sms), 256, 0, s>>>(tokens, tb, n, d->keys, d->cap - 1, limit,
+    k_dict_tokens<<<grid_for((n + 3) / 4, 256, c->num_sms), 256, 0, s>>>(tokens, tb, n, d->keys, d->cap - 1, limit,
                                                                misc + kMiscDict, misc + kMiscDict + 1);
   }
   if (!capturing(c))  // read in dictionary_finish (a captured call takes it from its tape there)
