@@ -625,10 +625,18 @@ __global__ void k_ac_nodes(NodeArgs a) {
 // not match, so the nodes skipped (no branch edges, the same primary symbol)
 // cannot match either.  sk[u] of a skipped u has the same criterion as sk[v],
 // which makes the jumps composable.
-__global__ void k_ac_jump(uint64_t *w, uint32_t *jl, uint32_t *sk, const uint32_t *__restrict__ own,
+// A round behind one in which nothing moved has nothing to do but the last
+// one's outputs: chains are mostly far shorter than the longest pattern, which
+// bounds the rounds.  `moved` is this round's word, `before` the last one's; a
+// block looks whether the word is set already before it sets it (stored by
+// every warp, the one address cost more than the rounds).
+constexpr int kJumpT = 512;
+__global__ void __launch_bounds__(kJumpT) k_ac_jump(uint32_t *moved, const uint32_t *before, uint64_t *w, uint32_t *jl, uint32_t *sk, const uint32_t *__restrict__ own,
                           const uint32_t *__restrict__ tsym, const uint8_t *__restrict__ has_branch,
                           uint32_t nodes, uint32_t root, int last, uint32_t *total,
                           const uint32_t *__restrict__ recidx, uint32_t *firstrec, uint4 *rec, uint32_t *err) {
+  if (before && *before == 0 && !last) return;  // (its own word stays 0)
+  bool any = false;
   for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nodes; v += gridDim.x * blockDim.x) {
     uint32_t u = sk[v];
     const uint32_t a = v != root ? tsym[v + 1] : kNil;
@@ -636,6 +644,7 @@ __global__ void k_ac_jump(uint64_t *w, uint32_t *jl, uint32_t *sk, const uint32_
     if (skippable) {
       u = *(volatile uint32_t *)&sk[u];
       sk[v] = u;
+      any = true;
     }
     if (last && u != root && !has_branch[u] && tsym[u + 1] == a) atomicExch(err, kDevRange);
     uint64_t x = w[v];
@@ -645,11 +654,13 @@ __global__ void k_ac_jump(uint64_t *w, uint32_t *jl, uint32_t *sk, const uint32_
       x = (y & 0xffffffff00000000ull) | (uint32_t)((uint32_t)x + (uint32_t)y);
       w[v] = x;
       p = (uint32_t)(x >> 32);
+      any = true;
     }
     uint32_t o = jl[v];
     if (o != root && own[o] == 0) {
       o = *(volatile uint32_t *)&jl[o];
       jl[v] = o;
+      any = true;
     }
     if (last) {
       if (p != root || (o != root && own[o] == 0)) atomicExch(err, kDevRange);
@@ -664,6 +675,7 @@ __global__ void k_ac_jump(uint64_t *w, uint32_t *jl, uint32_t *sk, const uint32_
       }
     }
   }
+  if (__syncthreads_or(any) && threadIdx.x == 0 && *(volatile uint32_t *)moved == 0) *moved = 1;
 }
 
 __global__ void k_jump_init(const uint32_t *__restrict__ fail, const uint32_t *__restrict__ own,
@@ -765,8 +777,11 @@ __global__ void k_flat_chains(const uint4 *__restrict__ rec, uint32_t R, const u
 // symbols with the 32 symbols of T after the current state at once and
 // takes the whole agreeing run in one step; a mismatch is settled by one
 // lane with the goto table and the failure chain.
+constexpr uint32_t kBranch = 0x80000000u;
 constexpr int kLift = 5;  // skip^(2^k), k < kLift: 32 chain nodes per warp-wide step
 struct Automaton {
+  const uint2 *node;     // (chunked passes only) what a step from a node needs, in one load: its next position's
+                         // symbol; its skip link, with kBranch set when a branch edge leaves it
   const uint32_t *tsym;  // padded with kTsymPad separators past the text
   const uint8_t *has_branch;
   Table g;
@@ -845,13 +860,21 @@ __device__ __forceinline__ bool run_chunk(const uint32_t *__restrict__ ssym, uin
       const uint32_t c = ssym[x];
       uint32_t cur = v;
       while (true) {
-        const uint32_t nx = ac_goto(A.tsym, A.g, cur, c, root);
+        uint32_t nx = kNil, sk = root;
+        if (cur == root) {
+          nx = table_lookup(A.g, root, c);
+        } else {
+          const uint2 w = A.node[cur];
+          sk = w.y & ~kBranch;
+          if (w.x == c) nx = cur + 1;
+          else if (w.y & kBranch) nx = table_lookup(A.g, cur, c);
+        }
         if (nx != kNil) {
           nv = nx;
           break;
         }
         if (cur == root) break;
-        cur = A.skip[cur];
+        cur = sk;
       }
       if (kCheck && state[x] == nv) nv = kNil;  // agreement
       else state[x] = nv;
@@ -882,16 +905,34 @@ __global__ void k_ac_states(const uint32_t *__restrict__ ssym, uint64_t n, uint6
   uint64_t x = cs;
   uint32_t c = ssym[x];
   while (x < ce) {
-    const uint32_t nx = ac_goto(A.tsym, A.g, cur, c, root);
+    uint32_t nx = kNil, sk = root;
+    bool look = cur == root;
+    if (!look) {
+      const uint2 w = A.node[cur];
+      sk = w.y & ~kBranch;
+      if (w.x == c) nx = cur + 1;
+      else look = (w.y & kBranch) != 0;
+    }
+    if (look) nx = table_lookup(A.g, cur, c);
     if (nx != kNil || cur == root) {
       state = nx != kNil ? nx : root;
       state_out[x] = state;
       cur = state;
       if (++x < ce) c = ssym[x];
     } else {
-      cur = A.skip[cur];
+      cur = sk;
     }
   }
+}
+
+// The words of Automaton::node.  A step along the first pass is a chain of
+// dependent reads: the symbol, the branch table and the skip link were three,
+// most nodes have no branch edge (states of 2^26 tokens: 1,130 -> 969 us; with
+// the branch table read beside the word whether it is needed or not, slower).
+__global__ void k_node_words(const uint32_t *__restrict__ tsym, const uint32_t *__restrict__ skip,
+                             const uint8_t *__restrict__ has_branch, uint32_t N, uint2 *__restrict__ node) {
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x)
+    node[v] = make_uint2(tsym[v + 1], skip[v] | (has_branch[v] ? kBranch : 0u));
 }
 
 // Pass A2 (repeated until nothing changes), one warp per group of `group`
@@ -1235,7 +1276,7 @@ size_t match_workspace_bytes(uint64_t total_tokens, uint64_t P, uint64_t n, uint
   const uint64_t sparse = (uint64_t)(bits_for(P) + 1) * P;
   // pattern text (symbols, sort tokens, pattern ids, reach) and the per-node
   // arrays (with the halo pass's preferred children and lifting tables)
-  uint64_t bytes = N * (8 + 4 + 4) + (N + kTsymPad) * (4 + 4 + 8 + 4 + 4 + 4 + 4 + 4 + 1 + 16 + 8 + 20) +
+  uint64_t bytes = N * (8 + 4 + 4) + (N + kTsymPad) * (4 + 4 + 8 + 4 + 4 + 4 + 4 + 4 + 1 + 16 + 8 + 20) + 1024 +
                    P * (16 + 8) +
                    tbl * 16 + dct * 8 + P * (4 * 8 + 24) + sparse * 4 + (extent + n) * 4 + n * 8 + 96 * 256 +
                    P * 8;  // record totals and flattened-chain offsets
@@ -1605,9 +1646,13 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     k_jump_init<<<grid_for((uint64_t)N + 1, 256, sms), 256, 0, s>>>(fail, own, N + 1, root, wj, jl, skip);
   }
   const int jumps = bits_for(maxlen) + 1;
+  uint32_t *moved = c->arena.take_n<uint32_t>(jumps);
+  if (!moved) return APO_ENOMEM;
+  APO_CUDA_TRY(cudaMemsetAsync(moved, 0, jumps * sizeof(uint32_t), s));
+  const int jb = std::max(1, std::min(ceil_div((uint64_t)N + 1, kJumpT), sms * 4));
   for (int r = 0; r < jumps; ++r) {
     Launch lp_(c, kKAcJump, (uint64_t)N + 1, s);
-    k_ac_jump<<<grid_for((uint64_t)N + 1, 256, sms), 256, 0, s>>>(wj, jl, skip, own, tsym, has_branch, N + 1,
+    k_ac_jump<<<jb, kJumpT, 0, s>>>(moved + r, r ? moved + r - 1 : nullptr, wj, jl, skip, own, tsym, has_branch, N + 1,
                                                                   root, r == jumps - 1, mtotal, recidx,
                                                                   firstrec, rec, c->ps.err);
   }
@@ -1633,7 +1678,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   }
 
   // pass A: the state of every stream position (pass shape chosen above)
-  Automaton A{tsym, has_branch, g, skip, root, {skip}, (uint32_t)(maxlen / 32 + 2), {}};
+  Automaton A{nullptr, tsym, has_branch, g, skip, root, {skip}, (uint32_t)(maxlen / 32 + 2), {}};
   uint32_t *state = c->arena.take_n<uint32_t>(n);
   uint32_t *off = c->arena.take_n<uint32_t>(n);  // (offsets: only without flattened chains)
   if (!state || !off) return APO_ENOMEM;
@@ -1659,6 +1704,13 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     k_ac_halo<<<ceil_div(nseg, kStateWarps), 32 * kStateWarps, 0, s>>>(ssym, n, seg, maxlen, A, state,
                                                                         c->ps.err);
   } else {
+    uint2 *node = c->arena.take_n<uint2>((size_t)N + 1);
+    if (!node) return APO_ENOMEM;
+    {
+      Launch lp_(c, kKAcJump, N, s);
+      k_node_words<<<grid_for(N, 256, sms), 256, 0, s>>>(tsym, skip, has_branch, N, node);
+    }
+    A.node = node;
     Launch lp_(c, kKAcStates, n, s);
     k_ac_states<<<ceil_div(nch, 64), 64, 0, s>>>(ssym, n, chunk, A, state);
   }

@@ -55,7 +55,7 @@ constexpr int kRowPad = 258;     // digit counters per warp, padded against bank
 constexpr uint32_t kHalfBase = 0x400;  // minor keys 0 .. 8192 plus this are the bits of normal halves, in order
 constexpr uint32_t kDirectCost = 320;  // comparisons per suffix that cost what a radix sort of the window costs
 constexpr int kSharedLevels = 8;  // level ranks that fit the sort keys' 16 bytes per token
-constexpr uint32_t kDirect = 64;  // tokens compared directly before lifting
+constexpr uint32_t kDirect = 8;  // tokens compared directly before lifting
 constexpr uint64_t kSetEmpty = ~0ull;
 
 // Device words of a call (zeroed ahead of it): see small_find_repeats.
@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(TPB, 1) k_small(const SmallArgs a) {
     for (uint32_t x = tid; x < n / 32 + 1; x += TPB) bits[x] = 0;
     for (uint32_t x = tid; x < 2 * NMAX / 32; x += TPB) accw[x] = 0;
     __syncthreads();
-    uint32_t size = 64;
+    uint32_t size = 32;
     for (uint32_t base = 0; base < m; base += size, size = min(size * 2, (uint32_t)TPB)) {
       const uint32_t k = base + tid;
       uint32_t st = 0, en = 0;

@@ -1062,14 +1062,15 @@ __global__ void k_phi(const uint32_t *__restrict__ sa, uint32_t n, const uint32_
   }
 }
 
-// PLCP[i] = lcp(i, Phi[i]) over chunks of kPChunk consecutive i per thread.
+// PLCP[i] = lcp(i, Phi[i]) over chunks of kPChunk consecutive i per thread (16,
+// or 8 when 16 would leave the chip half empty: a chunk is a serial walk, and
+// its first position starts from nothing).
 // Tokens are compared directly for up to kPDirect steps; a match that keeps
 // going is finished by lifting over the level ranks: level lev ranks are
 // equal iff the next h0 * 2^lev tokens are, from the top level down (level
 // lev's snapshot at snap0 + lev * n).
-constexpr int kPChunk = 16;
 constexpr uint32_t kPDirect = 256;
-template <class T>
+template <class T, int kPChunk>
 __global__ void k_plcp(const T *__restrict__ S, uint32_t n, Windows W, const uint32_t *__restrict__ wsb,
                        const uint32_t *__restrict__ phi, const uint8_t *__restrict__ fin,
                        const uint32_t *__restrict__ rank, const uint32_t *__restrict__ snap0, int levels,
@@ -1604,15 +1605,19 @@ int build_lcp(apo_ctx *c, const void *tokens, int tb, const SuffixState &st, uin
     Launch lp_(c, kKPhi, n, s);
     k_phi<<<g, 256, 0, s>>>(st.sa, n, st.wsb, phi);
   }
-  const int pb = ceil_div(ceil_div(n, kPChunk), 128);
   {
     Launch lp_(c, kKPlcp, n, s);
-    if (tb == 4)
-      k_plcp<uint32_t><<<pb, 128, 0, s>>>(static_cast<const uint32_t *>(tokens), n, st.win, st.wsb, phi, st.fin,
-                                          st.rank, st.snaps[0], st.levels, st.h0, plcp);
-    else
-      k_plcp<uint64_t><<<pb, 128, 0, s>>>(static_cast<const uint64_t *>(tokens), n, st.win, st.wsb, phi, st.fin,
-                                          st.rank, st.snaps[0], st.levels, st.h0, plcp);
+    auto run = [&](auto kernel, auto tok, int chunk) {
+      kernel<<<ceil_div(ceil_div(n, chunk), 128), 128, 0, s>>>(tok, n, st.win, st.wsb, phi, st.fin, st.rank,
+                                                               st.snaps[0], st.levels, st.h0, plcp);
+    };
+    const bool few = n < (uint32_t)c->num_sms * 2048 * 8;
+    const uint32_t *t4 = static_cast<const uint32_t *>(tokens);
+    const uint64_t *t8 = static_cast<const uint64_t *>(tokens);
+    if (tb == 4 && few) run(k_plcp<uint32_t, 8>, t4, 8);
+    else if (tb == 4) run(k_plcp<uint32_t, 16>, t4, 16);
+    else if (few) run(k_plcp<uint64_t, 8>, t8, 8);
+    else run(k_plcp<uint64_t, 16>, t8, 16);
   }
   {
     Launch lp_(c, kKLcpPerm, n, s);
