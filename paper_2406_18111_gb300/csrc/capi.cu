@@ -395,10 +395,11 @@ __global__ void __launch_bounds__(256) k_fill_windows(const uint32_t *__restrict
   }
 }
 
+// (a window's suffixes occupy its own slots: the window is read at the slot)
 __global__ void k_sa_relative(const uint32_t *__restrict__ sa, uint32_t n, const uint32_t *__restrict__ wid,
                               const uint32_t *__restrict__ off, uint32_t *__restrict__ out) {
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-    out[k] = sa[k] - off[wid[sa[k]]];
+    out[k] = sa[k] - off[wid[k]];
 }
 
 // Shared driver of apo_find_repeats (one window) and apo_find_repeats_batched.

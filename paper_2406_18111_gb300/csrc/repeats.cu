@@ -243,27 +243,30 @@ __global__ void __launch_bounds__(kCT) k_compact(Pred pred, uint32_t m, const ui
   }
 }
 
-__global__ void k_cand_gather(const uint32_t *__restrict__ sel, uint32_t m, const uint32_t *m_dev,
-                              const uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
-                              int bi, int bl, uint32_t lmax, int ks, const uint32_t *__restrict__ woff,
-                              uint32_t nwin, uint32_t *__restrict__ cl, uint32_t *__restrict__ cid,
-                              uint32_t *__restrict__ cs, uint32_t *err) {
-  m = min(m, *m_dev);  // m: an upper bound
-  const uint64_t idmask = (bi >= 64) ? ~0ull : ((1ull << bi) - 1);
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
-    const uint32_t k = sel[q];
+// The r-th candidate left by the deduplication, decoded from its key (and
+// value, when the key does not hold the start) to global positions.
+struct PutCand {
+  const uint64_t *keys;
+  const uint32_t *vals;
+  int bi, bl, ks;
+  uint32_t lmax;
+  const uint32_t *woff;
+  uint32_t nwin;
+  uint32_t *cl, *cid, *cs, *err;
+  __device__ __forceinline__ void operator()(uint32_t r, uint32_t k) const {
+    const uint64_t idmask = (bi >= 64) ? ~0ull : ((1ull << bi) - 1);
     const uint64_t full = keys[k], key = full >> ks;
     const uint64_t w = key >> (bl + bi);
     if (woff && w >= nwin) {  // (only keys of a replay whose checks failed)
       atomicExch(err, kDevRange);
-      continue;
+      return;
     }
-    const uint32_t base = woff ? woff[(uint32_t)w] : 0u;  // back to global positions
-    cl[q] = lmax - (uint32_t)((key >> bi) & lmax);
-    cid[q] = (uint32_t)(key & idmask) + base;
-    cs[q] = (ks ? (uint32_t)(full & ((1ull << ks) - 1)) : vals[k]) + base;
+    const uint32_t base = woff ? woff[(uint32_t)w] : 0u;
+    cl[r] = lmax - (uint32_t)((key >> bi) & lmax);
+    cid[r] = (uint32_t)(key & idmask) + base;
+    cs[r] = (ks ? (uint32_t)(full & ((1ull << ks) - 1)) : vals[k]) + base;
   }
-}
+};
 
 // ---------------------------------------------------------------- greedy
 constexpr int kGI = 4;  // candidates per thread per round
@@ -885,14 +888,10 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int tb, const SuffixSta
       APO_TRY(radix_sort_planned(c, b, mraw, sp, s, nullptr, true));
     }
     PredFirstOfRun pr{b.keys[b.cur], ks ? nullptr : b.vals[b.cur]};
-    APO_TRY(compact(c, pr, mraw, sel, misc + kMiscCandUnique, s));
+    PutCand put{b.keys[b.cur], b.vals[b.cur], bi, bl, ks, lmax, W.count > 1 ? W.off_dev : nullptr,
+                W.count, cl, cid, cs, c->ps.err};
+    APO_TRY(compact_to(c, pr, put, mraw, misc + kMiscCandUnique, s));
     mu = mraw;
-    {
-      Launch lp_(c, kKCandGather, mu, s);
-      k_cand_gather<<<grid_for(mu, 256, c->num_sms), 256, 0, s>>>(sel, mu, m_dev, b.keys[b.cur], b.vals[b.cur],
-                                                                  bi, bl, lmax, ks, W.count > 1 ? W.off_dev : nullptr,
-                                                                  W.count, cl, cid, cs, c->ps.err);
-    }
   }
 
   // greedy selection, one block per window
