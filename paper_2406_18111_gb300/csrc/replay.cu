@@ -590,14 +590,18 @@ __global__ void __launch_bounds__(kSelectThreads)
 }
 
 // ---------------------------------------------------------------- outputs
-// One warp per replay: the replay record, the traced tasks, the traced total.
-__global__ void k_replay_out(uint32_t R, const uint32_t *__restrict__ chain, const uint32_t *__restrict__ winner,
-                             const uint32_t *__restrict__ plen, const uint32_t *__restrict__ upid,
-                             uint32_t *rep_end, uint32_t *rep_len,
-                             uint32_t *rep_trace, uint64_t rcap, uint8_t *traced,
-                             unsigned long long *traced_total, uint32_t *err) {
+// One warp per replay: the replay record, the traced tasks, the traced total
+// (summed per block first: one addition per replay queued on the one address).
+constexpr int kOutT = 256;
+__global__ void __launch_bounds__(kOutT)
+    k_replay_out(uint32_t R, const uint32_t *__restrict__ chain, const uint32_t *__restrict__ winner,
+                 const uint32_t *__restrict__ plen, const uint32_t *__restrict__ upid, uint32_t *rep_end,
+                 uint32_t *rep_len, uint32_t *rep_trace, uint64_t rcap, uint8_t *traced,
+                 unsigned long long *traced_total, uint32_t *err) {
+  __shared__ unsigned long long s_sum[kOutT / 32];
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  unsigned long long sum = 0;
   for (uint64_t r = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; r < R; r += warps) {
     const uint32_t w = winner[r], e = chain[r + 1] - 1;
     if (w == kNone) {  // no winner: the selection gave up (error word set) or a task had no candidate
@@ -611,10 +615,16 @@ __global__ void k_replay_out(uint32_t R, const uint32_t *__restrict__ chain, con
         rep_len[r] = L;
         rep_trace[r] = upid[w];
       }
-      atomicAdd(traced_total, (unsigned long long)L);
     }
+    sum += L;
     if (traced)
       for (uint32_t j = lane; j < L; j += 32) traced[e + 1 - L + j] = 1;
+  }
+  if (lane == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kOutT / 32; ++w) sum += s_sum[w];
+    if (sum) atomicAdd(traced_total, sum);
   }
 }
 
@@ -993,7 +1003,7 @@ int replay_stream(apo_ctx *c, const void *tokens, uint64_t n, int tb, const apo_
     }
     {
       Launch lp_(c, kKRpOut, R, s);
-      k_replay_out<<<grid_for((uint64_t)R * 32, 256, sms), 256, 0, s>>>(R, chain, w.winner, plen, upid, out->rep_end,
+      k_replay_out<<<grid_for((uint64_t)R * 32, kOutT, sms), kOutT, 0, s>>>(R, chain, w.winner, plen, upid, out->rep_end,
                                                                         out->rep_len, out->rep_trace, out->rep_cap,
                                                                         traced, traced_total, c->ps.err);
     }
