@@ -286,9 +286,10 @@ __device__ __forceinline__ bool marked(const uint32_t *bits, uint32_t x) {
 
 // One block per window runs Alg. 2's second loop over the window's
 // candidates [cand_off[w], cand_off[w+1]).  Each round takes the next kT * 4
-// candidates (base + i*kT + tid for item i of thread tid), drops those whose
-// first or last position is already marked, compacts the rest in candidate
-// order, and warp 0 settles them 32 at a time, marking accepted intervals.
+// candidates (warp w takes 128 consecutive ones, 32 per item), drops those
+// whose first or last position is already marked, compacts the rest in
+// candidate order, and warp 0 settles them 32 at a time, marking accepted
+// intervals.
 // The accepted flags must be zero on entry.  The mark bitmap covers the
 // window in shared memory (positions relative to the window start), or all
 // positions in global memory (zeroed by the caller).
@@ -323,15 +324,16 @@ __global__ void __launch_bounds__(kT) k_greedy(const uint32_t *__restrict__ cl,
   acc += cb;
   m = ce - cb;
   uint32_t *sl = gsm + words, *ss = sl + kGRound, *sk = ss + kGRound, *sov = sk + kGRound;
-  __shared__ uint32_t s_cnt[2][kGI][32];  // survivors per (item, warp), by round parity
+  __shared__ uint32_t s_cnt[2][32];  // survivors per warp, by round parity
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t mine0 = warp * (32 * kGI) + lane;  // the thread's first candidate of a round
   if (kSmem)
     for (uint32_t x = tid; x < words; x += kGT) gsm[x] = persist ? gbits[x] : 0u;
   uint32_t nacc = 0;
   uint32_t nl[kGI], ns[kGI], no[kGI];  // the next round's candidates, loaded a round ahead
 #pragma unroll
   for (int i = 0; i < kGI; ++i) {
-    const uint32_t k = i * kGT + tid;
+    const uint32_t k = mine0 + i * 32;
     nl[i] = k < m ? cl[k] : 0u;
     ns[i] = k < m ? cs[k] : 0u;
     no[i] = corig && k < m ? corig[k] : k;
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kT) k_greedy(const uint32_t *__restrict__ cl,
       l[i] = nl[i];
       s[i] = ns[i];
       o[i] = no[i];
-      const uint64_t kn = (uint64_t)base + kGRound + i * kGT + tid;  // prefetch the next round
+      const uint64_t kn = (uint64_t)base + kGRound + mine0 + i * 32;  // prefetch the next round
       if (kn < m) {
         nl[i] = cl[kn];
         ns[i] = cs[kn];
@@ -355,7 +357,7 @@ __global__ void __launch_bounds__(kT) k_greedy(const uint32_t *__restrict__ cl,
     }
 #pragma unroll
     for (int i = 0; i < kGI; ++i) {
-      const uint32_t k = base + i * kGT + tid;
+      const uint32_t k = base + mine0 + i * 32;
       surv[i] = false;
       if (k < m) {
         if (l[i] == 0 || s[i] < ws || (uint64_t)s[i] + l[i] > we) {
@@ -366,46 +368,55 @@ __global__ void __launch_bounds__(kT) k_greedy(const uint32_t *__restrict__ cl,
         }
       }
       bal[i] = __ballot_sync(0xffffffffu, surv[i]);
-      if (lane == 0) s_cnt[par][i][warp] = __popc(bal[i]);
+    }
+    {
+      uint32_t c = 0;
+#pragma unroll
+      for (int i = 0; i < kGI; ++i) c += __popc(bal[i]);
+      if (lane == 0) s_cnt[par][warp] = c;
     }
     __syncthreads();
-    // Survivor offsets in (item, warp) order = candidate order, scanned by
+    // Survivor offsets in (warp, item) order = candidate order, scanned by
     // every warp for itself.  The counts are double-buffered by round
     // parity: a round without survivors skips the barriers below, and a
     // warp may write the next round's counts while another still reads these.
-    uint32_t off[kGI], s_total = 0;
-#pragma unroll
-    for (int i = 0; i < kGI; ++i) {
-      const uint32_t c = lane < kGT / 32 ? s_cnt[par][i][lane] : 0u;
-      const uint32_t inc = warp_inclusive(c, OpSum());
-      off[i] = s_total + __shfl_sync(0xffffffffu, inc - c, warp);
-      s_total += __shfl_sync(0xffffffffu, inc, 31);
-    }
+    const uint32_t wc = lane < kGT / 32 ? s_cnt[par][lane] : 0u;
+    const uint32_t winc = warp_inclusive(wc, OpSum());
+    const uint32_t s_total = __shfl_sync(0xffffffffu, winc, 31);
     if (s_total == 0) continue;  // the same in every warp; no mark changes
+    uint32_t off = __shfl_sync(0xffffffffu, winc - wc, warp);
     const uint32_t lt = lanemask_lt();
 #pragma unroll
     for (int i = 0; i < kGI; ++i) {
       if (surv[i]) {
-        const uint32_t q = off[i] + __popc(bal[i] & lt);
+        const uint32_t q = off + __popc(bal[i] & lt);
         sl[q] = l[i];
         ss[q] = s[i];
         sk[q] = o[i];
       }
+      off += __popc(bal[i]);
     }
     __syncthreads();
     // Overlap masks of the survivor batches, by every warp (they depend on
     // the intervals only): sov[q] bit j = survivor q0 + j of q's batch of 32
     // (q0 = q rounded down to 32), j before q's lane, meets survivor q.
-    for (uint32_t q = tid; q < s_total; q += kGT) {
-      const uint32_t q0 = q & ~31u, nb = min(32u, s_total - q0);
-      const uint32_t qs = ss[q], qe = qs + sl[q] - 1;
+    // Four threads per survivor, eight comparisons each (a round has a few
+    // hundred survivors at most, the block 1,024 threads).
+    for (uint32_t g = tid & ~31u; g < 4 * s_total; g += kGT) {
+      const uint32_t q = (g + lane) >> 2, part = (lane & 3) * 8;
       uint32_t ov = 0;
+      if (q < s_total) {
+        const uint32_t q0 = q & ~31u, at = q & 31u;  // earlier survivors of the batch: j < at
+        const uint32_t qs = ss[q], qe = qs + sl[q] - 1;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const uint32_t js = ss[q0 + j], je = js + sl[q0 + j] - 1;  // list has room past total
-        if (j < lane && (uint32_t)j < nb && js <= qe && qs <= je) ov |= 1u << j;
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t p = part + j, js = ss[q0 + p], je = js + sl[q0 + p] - 1;  // the list has room past total
+          if (p < at && js <= qe && qs <= je) ov |= 1u << p;
+        }
       }
-      sov[q] = ov;
+      ov |= __shfl_xor_sync(0xffffffffu, ov, 1);
+      ov |= __shfl_xor_sync(0xffffffffu, ov, 2);
+      if (q < s_total && (lane & 3) == 0) sov[q] = ov;
     }
     __syncthreads();
     if (warp == 0 && s_total) {
