@@ -35,6 +35,10 @@ namespace {
 constexpr int kHistThreads = 256;
 constexpr int kMaxRadix = 512;
 constexpr int kMaxPass = 12;
+constexpr int kCtrSortEnd = kCtrSortBuf + kMaxPass + 1;  // the sort's counters from kCtrSortHist on
+static_assert(kCtrSortHist == 0 && kCtrSortTiles == kMaxPass * kMaxRadix && kCtrSortTiles + kMaxPass <= kCtrSortBuf &&
+                  kCtrSortEnd <= kCtrMisc,
+              "the sort's counters are cleared in one piece");
 
 struct Places {
   int p[kMaxPass];
@@ -88,6 +92,36 @@ struct PassShape {
   static_assert(kTile <= 65535, "per-warp digit prefixes are 16-bit");
 };
 
+// Adds the digits at next_place of the block's tile of keys into next_cnt.
+template <int TPB, int ITEMS, int BITS>
+__device__ __noinline__ void count_next(const uint64_t *kin, uint32_t n, int next_place, uint32_t *next_cnt) {
+  constexpr int R = 1 << BITS;
+  __shared__ uint32_t cnt[R];
+  const uint64_t base = (uint64_t)blockIdx.x * (TPB * ITEMS);
+  if (next_place < 0 || base >= n) return;
+  if (threadIdx.x < R) cnt[threadIdx.x] = 0;
+  __syncthreads();
+  uint64_t k[ITEMS];
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint64_t i = base + j * TPB + threadIdx.x;
+    k[j] = i < n ? kin[i] : 0;
+  }
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const bool valid = base + j * TPB + threadIdx.x < n;
+    const uint32_t d = valid ? digit_of<BITS>(k[j], 0u, next_place) : (uint32_t)R;
+    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+    if (__all_sync(0xffffffffu, d == d0 && d0 < (uint32_t)R)) {
+      if ((threadIdx.x & 31) == 0) atomicAdd(&cnt[d0], 32u);
+    } else if (valid) {
+      atomicAdd(&cnt[d], 1u);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < R && cnt[threadIdx.x]) atomicAdd(&next_cnt[threadIdx.x], cnt[threadIdx.x]);
+}
+
 // One digit place.  `gcnt` is this place's global digit histogram (the
 // tile turns it into digit offsets itself); when next_place >= 0 the tile
 // also counts the next place's digits of its keys into next_cnt, so no
@@ -102,10 +136,30 @@ __global__ void __launch_bounds__(TPB, (KO ? 1536 : 1024) / TPB) k_rs_pass(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint64_t *__restrict__ kout,
     uint32_t *__restrict__ vout, uint32_t n, const uint32_t *__restrict__ n_dev, int place,
     const uint32_t *__restrict__ gcnt, int next_place, uint32_t *__restrict__ next_cnt, uint64_t *status,
-    uint32_t *tile_ctr, uint32_t epoch, uint32_t *err) {
+    uint32_t *tile_ctr, uint32_t epoch, uint32_t *err, uint32_t *buf) {
   using S = PassShape<TPB, ITEMS, BITS, KO>;
   if (n_dev) n = min(n, *n_dev);  // the launch is sized for an upper bound
   constexpr int R = S::kRadix, NW = S::kWarps, TILE = S::kTile;
+  if (buf) {
+    // A sort that may skip places: *buf says which buffer holds the pairs
+    // before this one.  When every key has the same digit there is nothing to
+    // move; only the next place's digits are counted.
+    const uint32_t f = *buf;
+    const int same = __syncthreads_or(threadIdx.x < R && gcnt[threadIdx.x] == n);
+    if (blockIdx.x == 0 && threadIdx.x == 0) buf[1] = same ? f : f ^ 1u;
+    if (f) {
+      const uint64_t *ki = kin;
+      kin = kout;
+      kout = const_cast<uint64_t *>(ki);
+      const uint32_t *vi = vin;
+      vin = vout;
+      vout = const_cast<uint32_t *>(vi);
+    }
+    if (same) {
+      count_next<TPB, ITEMS, BITS>(kin, n, next_place, next_cnt);
+      return;
+    }
+  }
   extern __shared__ __align__(16) uint8_t smem[];
   uint64_t *sk = reinterpret_cast<uint64_t *>(smem);
   uint32_t *sv = reinterpret_cast<uint32_t *>(sk + TILE);  // (pairs only)
@@ -286,7 +340,8 @@ __global__ void k_rs_trial_keys(uint64_t *keys, uint32_t *vals, uint32_t n, int 
 
 // ---------------------------------------------------------------- shapes
 using PassFn = void (*)(const uint64_t *, const uint32_t *, uint64_t *, uint32_t *, uint32_t, const uint32_t *,
-                        int, const uint32_t *, int, uint32_t *, uint64_t *, uint32_t *, uint32_t, uint32_t *);
+                        int, const uint32_t *, int, uint32_t *, uint64_t *, uint32_t *, uint32_t, uint32_t *,
+                        uint32_t *);
 using HistFn = void (*)(const uint64_t *, const uint32_t *, uint32_t, const uint32_t *, int, uint32_t *);
 
 struct Shape {
@@ -321,7 +376,7 @@ int plan(const Shape &sh, const DigitRange *ranges, int nranges, Places *pl) {
 
 // All passes of one sort with one shape (b.cur flips once per pass).
 int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uint32_t *n_dev, const Places &pl,
-              bool count, cudaStream_t s, bool hist_ready = false) {
+              bool count, cudaStream_t s, bool hist_ready = false, uint32_t *buf = nullptr) {
   const int R = 1 << sh.bits;
   const int tile = sh.threads * sh.items;
   const int tiles = ceil_div(n, tile);
@@ -329,9 +384,9 @@ int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uin
   uint32_t *hist = c->ps.counters + kCtrSortHist;   // [kMaxPass][kMaxRadix]
   uint32_t *tctr = c->ps.counters + kCtrSortTiles;  // [kMaxPass]
   if (hist_ready) {  // the first place's counts are in; clear the others and the tile tickets
-    APO_CUDA_TRY(cudaMemsetAsync(hist + kMaxRadix, 0, ((kMaxPass - 1) * kMaxRadix + kMaxPass) * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(hist + kMaxRadix, 0, (kCtrSortEnd - kMaxRadix) * sizeof(uint32_t), s));
   } else {
-    APO_CUDA_TRY(cudaMemsetAsync(hist, 0, (kMaxPass * kMaxRadix + kMaxPass) * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(hist, 0, kCtrSortEnd * sizeof(uint32_t), s));
     const int hblocks = std::max(1, std::min(c->num_sms * 4, ceil_div(n, kHistThreads * 8)));
     Launch lp_(c, count ? kKRsHist : kKRsTune, n, s);
     sh.hist<<<hblocks, kHistThreads, 0, s>>>(b.keys[b.cur], b.vals[b.cur], n, n_dev, pl.p[0], hist);
@@ -346,9 +401,9 @@ int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uin
           b.keys[b.cur], b.vals[b.cur], b.keys[b.cur ^ 1],
                                                  b.vals[b.cur ^ 1], n, n_dev, pl.p[p], hist + p * kMaxRadix, nxt,
                                                  hist + (p + 1) * kMaxRadix, c->ps.lookback, tctr + p, ep,
-                                                 c->ps.err);
+                                                 c->ps.err, buf ? buf + p : nullptr);
     }
-    b.cur ^= 1;
+    if (!buf) b.cur ^= 1;
   }
   APO_CUDA_TRY(cudaGetLastError());
   return APO_OK;
@@ -508,6 +563,21 @@ int radix_sort_planned(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &s
   pl.n = sp.places;
   for (int p = 0; p < sp.places; ++p) pl.p[p] = sp.place[p];
   return sort_with(c, kShapes[sp.shape], b, n, n_dev, pl, true, s, hist_ready);
+}
+
+int radix_sort_skipping(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &sp, cudaStream_t s,
+                        const uint32_t *n_dev, const uint32_t **buf) {
+  uint32_t *w = c->ps.counters + kCtrSortBuf;
+  *buf = w + std::max(0, sp.places);
+  b.cur = 0;
+  if (sp.shape < 0) {  // nothing to sort: buffer 0
+    *buf = nullptr;
+    return APO_OK;
+  }
+  Places pl;
+  pl.n = sp.places;
+  for (int p = 0; p < sp.places; ++p) pl.p[p] = sp.place[p];
+  return sort_with(c, kShapes[sp.shape], b, n, n_dev, pl, true, s, true, w);
 }
 
 int radix_sort_pairs(apo_ctx *c, SortBuffers &b, uint32_t n, const DigitRange *ranges, int nranges,

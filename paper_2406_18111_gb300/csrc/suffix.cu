@@ -158,8 +158,12 @@ __global__ void __launch_bounds__(kST) k_split(
     int finals, uint32_t *__restrict__ snap, uint32_t *__restrict__ sa, uint32_t *__restrict__ rank,
     uint8_t *__restrict__ fin, uint32_t *__restrict__ nid, uint32_t *__restrict__ nhd, uint32_t list_cap,
     uint32_t *count_out, uint32_t n, uint64_t *st_max, uint64_t *st_sum, uint32_t *tile_ctr, uint32_t epoch,
-    uint32_t *err, int id_bits) {
+    uint32_t *err, int id_bits, const uint64_t *keys1, const uint32_t *vals1, const uint32_t *buf) {
   constexpr int NW = kST / 32;
+  if (buf && *buf) {  // the sort left its result in the other buffer
+    keys = keys1;
+    vals = vals1;
+  }
   __shared__ uint32_t s_tile, s_pmax, s_psum, s_scan[2 * NW];
   WarpScan<NW> scan{s_scan, 0};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1154,7 +1158,8 @@ int split_launch(apo_ctx *c, bool big, const uint64_t *keys, const uint32_t *val
                  const uint32_t *n_dev, int ord_shift, const uint32_t *bg_head, const uint32_t *bg_off,
                  const uint32_t *bg_pos, uint32_t bg_cap, uint32_t level, bool finals, uint32_t *snap,
                  SuffixState &st, uint32_t *nid, uint32_t *nhd, uint32_t *count_out, cudaStream_t s,
-                 int id_bits = 0) {
+                 int id_bits = 0, const uint64_t *keys1 = nullptr, const uint32_t *vals1 = nullptr,
+                 const uint32_t *buf = nullptr) {
   const int tiles = std::max(1, ceil_div(ub, kSTile));
   APO_TRY(ensure_lookback(c, (size_t)2 * tiles));
   uint32_t *misc = c->ps.counters + kCtrMisc;
@@ -1165,12 +1170,12 @@ int split_launch(apo_ctx *c, bool big, const uint64_t *keys, const uint32_t *val
     k_split<true><<<tiles, kST, 0, s>>>(keys, vals, ub, n_dev, ord_shift, bg_head, bg_off, bg_pos, bg_cap, level,
                                         finals, snap, st.sa, st.rank, st.fin, nid, nhd, st.n, count_out, st.n,
                                         c->ps.lookback, c->ps.lookback + tiles, misc + kMiscRefreshTiles, ep,
-                                        c->ps.err, id_bits);
+                                        c->ps.err, id_bits, keys1, vals1, buf);
   else
     k_split<false><<<tiles, kST, 0, s>>>(keys, vals, ub, n_dev, 0, nullptr, nullptr, nullptr, 0, level, finals,
                                          snap, st.sa, st.rank, st.fin, nid, nhd, st.n, count_out, st.n,
                                          c->ps.lookback, c->ps.lookback + tiles, misc + kMiscRefreshTiles, ep,
-                                         c->ps.err, 0);
+                                         c->ps.err, 0, nullptr, nullptr, nullptr);
   APO_CUDA_TRY(cudaGetLastError());
   return APO_OK;
 }
@@ -1523,9 +1528,12 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
       SortBuffers bb = b;
       bb.cur = 0;
       if (id_bits) bb.vals[0] = bb.vals[1] = nullptr;
-      APO_TRY(radix_sort_planned(c, bb, big_ub, sp, s, words + 1, true));
-      APO_TRY(split_launch(c, true, bb.keys[bb.cur], bb.vals[bb.cur], big_ub, words + 1, mb, bg_head, bg_off,
-                           bg_pos, bg_cap, r, true, st.snaps[r], st, hid, hhd, nullptr, s, id_bits));
+      // the ordinals' bits are sized for as many big groups as the entries
+      // could form; with few and large ones (runs) whole digits are zero
+      const uint32_t *buf = nullptr;
+      APO_TRY(radix_sort_skipping(c, bb, big_ub, sp, s, words + 1, &buf));
+      APO_TRY(split_launch(c, true, bb.keys[0], bb.vals[0], big_ub, words + 1, mb, bg_head, bg_off, bg_pos, bg_cap,
+                           r, true, st.snaps[r], st, hid, hhd, nullptr, s, id_bits, bb.keys[1], bb.vals[1], buf));
     }
     APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscRoundTiles, 0, sizeof(uint32_t), s));
     {
