@@ -131,7 +131,7 @@ __device__ __noinline__ void count_next(const uint64_t *kin, uint32_t n, int nex
 // is loaded by the threads.  KO: keys only (vin, vout unused; no value
 // digits).  Without values a thread needs fewer registers and a tile less
 // shared memory, so three blocks of 512 threads fit an SM instead of two.
-template <int TPB, int ITEMS, int BITS, bool KO>
+template <int TPB, int ITEMS, int BITS, bool KO, bool SKIP>
 __global__ void __launch_bounds__(TPB, (KO ? 1536 : 1024) / TPB) k_rs_pass(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint64_t *__restrict__ kout,
     uint32_t *__restrict__ vout, uint32_t n, const uint32_t *__restrict__ n_dev, int place,
@@ -140,8 +140,9 @@ __global__ void __launch_bounds__(TPB, (KO ? 1536 : 1024) / TPB) k_rs_pass(
   using S = PassShape<TPB, ITEMS, BITS, KO>;
   if (n_dev) n = min(n, *n_dev);  // the launch is sized for an upper bound
   constexpr int R = S::kRadix, NW = S::kWarps, TILE = S::kTile;
-  if (buf) {
-    // A sort that may skip places: *buf says which buffer holds the pairs
+  if (SKIP) {
+    // A sort that may skip places (an instantiation of its own: the others
+    // lose 4% to the two reads ahead of everything else): *buf says which buffer holds the pairs
     // before this one.  When every key has the same digit there is nothing to
     // move; only the next place's digits are counted.
     const uint32_t f = *buf;
@@ -346,15 +347,16 @@ using HistFn = void (*)(const uint64_t *, const uint32_t *, uint32_t, const uint
 
 struct Shape {
   int threads, items, bits;
-  PassFn pass, pass_keys;  // (key, value) pairs; keys only
+  PassFn pass[2], pass_keys[2];  // (key, value) pairs; keys only; [1]: may skip places
   HistFn hist;
   size_t smem, smem_keys;
 };
 
 template <int TPB, int ITEMS, int BITS>
 constexpr Shape shape() {
-  return Shape{TPB, ITEMS, BITS, k_rs_pass<TPB, ITEMS, BITS, false>, k_rs_pass<TPB, ITEMS, BITS, true>,
-               k_rs_hist<BITS>, PassShape<TPB, ITEMS, BITS, false>::kSmem, PassShape<TPB, ITEMS, BITS, true>::kSmem};
+  return Shape{TPB, ITEMS, BITS, {k_rs_pass<TPB, ITEMS, BITS, false, false>, k_rs_pass<TPB, ITEMS, BITS, false, true>},
+               {k_rs_pass<TPB, ITEMS, BITS, true, false>, k_rs_pass<TPB, ITEMS, BITS, true, true>}, k_rs_hist<BITS>,
+               PassShape<TPB, ITEMS, BITS, false>::kSmem, PassShape<TPB, ITEMS, BITS, true>::kSmem};
 }
 
 // Shape 0 is the default (and the only one used with tuning off).
@@ -397,7 +399,7 @@ int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uin
     {
       const bool ko = b.vals[b.cur] == nullptr;
       Launch lp_(c, count ? (ko ? kKRsPassKeys : kKRsPass) : kKRsTune, n, s);
-      (ko ? sh.pass_keys : sh.pass)<<<tiles, sh.threads, ko ? sh.smem_keys : sh.smem, s>>>(
+      (ko ? sh.pass_keys : sh.pass)[buf != nullptr]<<<tiles, sh.threads, ko ? sh.smem_keys : sh.smem, s>>>(
           b.keys[b.cur], b.vals[b.cur], b.keys[b.cur ^ 1],
                                                  b.vals[b.cur ^ 1], n, n_dev, pl.p[p], hist + p * kMaxRadix, nxt,
                                                  hist + (p + 1) * kMaxRadix, c->ps.lookback, tctr + p, ep,
@@ -413,10 +415,12 @@ int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uin
 
 int radix_sort_init() {
   for (int i = 0; i < kNumShapes; ++i) {
-    APO_CUDA_TRY(cudaFuncSetAttribute((const void *)kShapes[i].pass,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShapes[i].smem));
-    APO_CUDA_TRY(cudaFuncSetAttribute((const void *)kShapes[i].pass_keys,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShapes[i].smem_keys));
+    for (PassFn f : kShapes[i].pass)
+      APO_CUDA_TRY(cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kShapes[i].smem));
+    for (PassFn f : kShapes[i].pass_keys)
+      APO_CUDA_TRY(cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kShapes[i].smem_keys));
   }
   return APO_OK;
 }
