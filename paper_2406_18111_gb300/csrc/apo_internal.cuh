@@ -79,6 +79,7 @@ enum : int {
   kMiscRoundTiles = 30,   // tile tickets of a doubling round
   kMiscRoundW = 32,       // 2 x 4 words of consecutive doubling rounds (see build_suffix_array)
   kMiscSmall = 48,        // 8 words of a small-window call (see small.cu)
+  kMiscDictHits = 56,     // tokens the dictionary held already when they came
   kMiscCount = 64,
 };
 

@@ -311,12 +311,16 @@ __device__ __forceinline__ uint64_t token_at(const void *tokens, int tb, uint32_
 // with one addition per new token, 2^22 of them (a window of random tokens,
 // where the dictionary is given up) queued on one address for 0.8 ms.
 __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t n, uint64_t *keys, uint64_t mask,
-                              uint32_t limit, uint32_t *distinct, uint32_t *over) {
+                              uint32_t limit, uint32_t *distinct, uint32_t *over, uint32_t *hits) {
+  __shared__ uint32_t s_hits;  // tokens found present, of those looked at before the dictionary was given up
+  if (threadIdx.x == 0) s_hits = 0;
+  __syncthreads();
+  uint32_t held = 0;
   constexpr int kI = 4;  // tokens per thread: their first slots' reads are under way together
   const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kI;
   for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kI; b0 < n; b0 += stride) {
-    if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) return;
+    if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) break;
     uint64_t t[kI], cur[kI];
     uint32_t fresh = 0;
 #pragma unroll
@@ -353,9 +357,16 @@ __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t 
         }
       }
     }
+#pragma unroll
+    for (int u = 0; u < kI; ++u) held += t[u] != kDictEmpty;
+    held -= fresh;
     const uint32_t c = __reduce_add_sync(0xffffffffu, fresh);
     if (lane == 0 && c && atomicAdd(distinct, c) + c > limit) atomicExch(over, 1u);
   }
+  held = __reduce_add_sync(0xffffffffu, held);
+  if (lane == 0 && held) atomicAdd(&s_hits, held);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_hits) atomicAdd(hits, s_hits);
 }
 
 // (token, slot) of every occupied slot, in any order (sorted next).
@@ -1198,6 +1209,7 @@ struct DictCodes {
   uint32_t *slot_code = nullptr, *codes = nullptr;
   SortBuffers lb;
   bool ok = false;
+  bool mostly_distinct = false;  // fewer than one token in nine had come before
 };
 
 int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCodes *d, cudaStream_t s) {
@@ -1215,13 +1227,17 @@ int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCod
   uint32_t *misc = c->ps.counters + kCtrMisc;
   APO_CUDA_TRY(cudaMemsetAsync(d->keys, 0xff, d->cap * sizeof(uint64_t), s));
   APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDict, 0, 2 * sizeof(uint32_t), s));
+  APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDictHits, 0, sizeof(uint32_t), s));
   {
     Launch lp_(c, kKSaDict, n, s);
     k_dict_tokens<<<grid_for((n + 3) / 4, 256, c->num_sms), 256, 0, s>>>(tokens, tb, n, d->keys, d->cap - 1, limit,
-                                                               misc + kMiscDict, misc + kMiscDict + 1);
+                                                               misc + kMiscDict, misc + kMiscDict + 1,
+                                                               misc + kMiscDictHits);
   }
-  if (!capturing(c))  // read in dictionary_finish (a captured call takes it from its tape there)
+  if (!capturing(c)) {  // read in dictionary_finish (a captured call takes it from its tape there)
     APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscDict, 8, cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 4, misc + kMiscDictHits, 4, cudaMemcpyDeviceToHost, s));
+  }
   return APO_OK;
 }
 
@@ -1231,13 +1247,24 @@ int dictionary_finish(apo_ctx *c, const void *tokens, int tb, uint32_t n, int tb
   uint32_t *misc = c->ps.counters + kCtrMisc;
   if (!d->ok) return APO_OK;
   uint32_t sv[2];  // distinct tokens, overflow flag
+  uint32_t few;    // most tokens are distinct (a choice of key length, not a result: taken from the tape unchecked)
   if (capturing(c)) {
     APO_TRY(tape_take(c, misc + kMiscDict, sv, 2, s));
+    if (c->tape->pos >= c->tape->vals.size()) {
+      set_error("graph capture: the call read more values than it recorded");
+      return APO_EDEVICE;
+    }
+    few = c->tape->vals[c->tape->pos++];
   } else {
     sv[0] = c->host_pinned[2];
     sv[1] = c->host_pinned[3];
-    if (recording(c)) tape_put(c, sv, 2);
+    few = (uint64_t)c->host_pinned[4] * 8 < sv[0];
+    if (recording(c)) {
+      tape_put(c, sv, 2);
+      tape_put(c, &few, 1);
+    }
   }
+  d->mostly_distinct = few != 0;
   const uint32_t sigma = sv[0];
   if (sv[1] || sigma > d->cap / 2) return APO_OK;
   APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDict, 0, sizeof(uint32_t), s));
@@ -1369,9 +1396,16 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
       h0 = (uint32_t)((64 - wb) / cb);
     }
   }
+  // Where a key would hold two tokens and nearly every token is distinct, the
+  // first token alone tells nearly all suffixes apart: half the digit places
+  // (2^24 random u32 tokens: four passes instead of eight), and a round over
+  // the few that are left.  Level L then stands for 2^L tokens instead of
+  // 2^(L+1); the rounds reported stay those of the two-token key, one fewer.
+  const bool one = h0 == 2 && dict.mostly_distinct;
+  if (one) h0 = 1;
   // level 0: groups of equal first h0 tokens (within a window)
   uint32_t *first_count = misc + kMiscRefreshCount;
-  if (h0 >= 2) {
+  if (h0 >= 2 || one) {
     h0 = std::min<uint32_t>(h0, 32);
     const DigitRange r{0, wb + (int)h0 * cb, false};
     SortPlan sp;
@@ -1594,7 +1628,7 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
     big_ub = std::min(big_ub, w2[1]);
     if (w2[1] == 0) big_possible = false;
   }
-  *rounds_out = (uint32_t)(st.levels - 1);
+  *rounds_out = (uint32_t)std::max(0, st.levels - 1 - (one ? 1 : 0));
   return APO_OK;
 }
 
