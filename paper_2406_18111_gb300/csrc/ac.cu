@@ -48,9 +48,9 @@
 // deterministic automaton repeats the recorded run.  When a pass changes no
 // end state all states are exact (after k passes groups 0..k are, by
 // induction); passes are queued two at a time, and one behind a pass without
-// changes returns at once.  The per-node match totals turn the output
-// offsets into one prefix sum over positions; each output record's chain is
-// flattened once, and a final kernel per position copies its matches.
+// changes returns at once.  Each output record's chain is flattened once, and
+// one kernel over the positions places their matches by a look-back sum of
+// the records' totals and copies the chains.
 // Where the patterns are slices of the stream itself and long (deep
 // states over much of the stream), one exact pass replaces the chunks and
 // repairs: a warp per segment starts its walk one longest-pattern length
@@ -103,14 +103,6 @@ __device__ __forceinline__ uint32_t table_lookup(const Table &g, uint32_t u, uin
     if (e.x == kEmpty) return kNil;
     slot = (slot + 1) & g.mask;
   }
-}
-
-// goto(v, c): the primary edge when T continues with c after v, else the
-// branch table.
-__device__ __forceinline__ uint32_t ac_goto(const uint32_t *__restrict__ tsym, const Table &g,
-                                            uint32_t v, uint32_t c, uint32_t root) {
-  if (v != root && tsym[v + 1] == c) return v + 1;
-  return table_lookup(g, v, c);
 }
 
 // ---------------------------------------------------------------- symbols
