@@ -66,7 +66,8 @@ struct SmallArgs {
   const uint32_t *off;     // [W + 1] window offsets, null for one window
   uint32_t W, n;           // windows; tokens of the single window
   uint32_t min_len;
-  uint16_t *snaps;         // level ranks: window w's level L at (off[w] * levels + L * n_w)
+  uint16_t *snaps;         // level ranks: window w's level L at (off[w] * levels, up to a multiple of 8) + 8 w + L * n_w
+                           // (16-byte boundaries, and no window reaches into the next one's)
   int levels;
   uint32_t *sa, *lcp;      // outputs as apo_repeats_out (null: not wanted)
   uint32_t *cl, *cid, *cs;
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(TPB, 1) k_small(const SmallArgs a) {
   const int nb = max(1, sm_bits(n ? n - 1 : 0));
   uint32_t m = 0, K = 0, Tn = 0;  // candidates, accepted, traces
   uint32_t maxl = 0;
-  uint16_t *snap = a.snaps + (((size_t)o0 * a.levels + 7) & ~(size_t)7);
+  uint16_t *snap = a.snaps + (((size_t)o0 * a.levels + 7) & ~(size_t)7) + (size_t)w * 8;
 
   if (n) {
     // ---- dense codes: the tokens in order
@@ -556,14 +557,9 @@ __global__ void __launch_bounds__(TPB, 1) k_small(const SmallArgs a) {
     // (the sorts are done: buf holds the first eight levels' ranks)
     uint16_t *lev_s = reinterpret_cast<uint16_t *>(buf);
     {
-      // (a window's ranks start anywhere: 16-byte copies from a 16-byte boundary where they do)
       const uint32_t total = n * (uint32_t)min(level + 1, kSharedLevels);
-      if ((reinterpret_cast<uintptr_t>(snap) & 15) == 0) {
-        for (uint32_t x = tid; x < (total + 7) / 8; x += TPB)
-          reinterpret_cast<uint4 *>(lev_s)[x] = reinterpret_cast<const uint4 *>(snap)[x];
-      } else {
-        for (uint32_t x = tid; x < total; x += TPB) lev_s[x] = snap[x];
-      }
+      for (uint32_t x = tid; x < (total + 7) / 8; x += TPB)
+        reinterpret_cast<uint4 *>(lev_s)[x] = reinterpret_cast<const uint4 *>(snap)[x];
     }
     __syncthreads();
     {
@@ -955,7 +951,7 @@ int small_find_repeats(apo_ctx *c, const void *tokens, int tb, const uint64_t *w
   a.n = total;
   a.min_len = p->min_len;
   a.levels = bits_for(longest) + 2;
-  a.snaps = c->arena.take_n<uint16_t>((size_t)total * a.levels + 16);
+  a.snaps = c->arena.take_n<uint16_t>((size_t)total * a.levels + 8 * (size_t)W + 16);
   bool ok = a.snaps != nullptr;
   uint32_t *off = nullptr;
   // the distinct tokens of all windows are counted for the rounds reported

@@ -42,6 +42,7 @@ def test_batches_equal_the_general_path(apo, tb, hi):
     from paper_2406_18111_gb300 import as_u32
     kinds = ("loop", "run", "few") if tb == 4 else ("tasks", "random", "loop")
     lens = np.r_[0, W.log_uniform_int(W.uniform01(hi, 60), 3, hi), hi, 0]
+    lens = np.insert(lens, np.arange(1, len(lens), 3), 1)  # one-token windows between the others
     wins = [window(kinds[w % 3], int(n), 900 + w) for w, n in enumerate(lens)]
 
     def run(ws):
