@@ -746,16 +746,34 @@ struct DstExclusive {  // out[k] = inclusive - a[k]; *sum = the grand total
   }
 };
 
-// One warp per record walks its chain and writes the ids.
+// The chains' total decides whether they are flattened and sizes the buffer,
+// and it can pass 2^32 (2^20 copies of a one-token pattern below 4,096 nested
+// ones): the sum stops at 2^32 - 1 instead of wrapping.
+struct OpSatSum {
+  __device__ __forceinline__ uint32_t operator()(uint32_t a, uint32_t b) const {
+    const uint32_t s = a + b;
+    return s < a ? 0xffffffffu : s;
+  }
+};
+
+// One warp per record walks its chain and writes the ids.  Nothing is written
+// behind an error (the records and links of an automaton that failed to build
+// can point anywhere), nor past the P ids or the buffer's `entries`.
 __global__ void k_flat_chains(const uint4 *__restrict__ rec, uint32_t R, const uint32_t *__restrict__ flat_off,
-                              const uint32_t *__restrict__ evals, uint32_t *__restrict__ flat) {
+                              const uint32_t *__restrict__ evals, uint32_t P, uint32_t *__restrict__ flat,
+                              uint64_t entries, uint32_t *err) {
+  if (*(volatile uint32_t *)err) return;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += warps) {
-    uint32_t o = flat_off[r];
+    uint64_t o = flat_off[r];
     uint32_t cur = r;
     while (cur != kNil) {
-      const uint4 q = rec[cur];
+      const uint4 q = cur < R ? rec[cur] : make_uint4(0, 0, kNil, 0);
+      if (q.y == 0 || (uint64_t)q.x + q.y > P || o + q.y > entries) {  // (every record ends a pattern)
+        if (lane == 0) atomicExch(err, kDevRange);
+        break;
+      }
       for (uint32_t k = lane; k < q.y; k += 32) flat[o + k] = evals[q.x + k];
       o += q.y;
       cur = q.z;
@@ -1161,8 +1179,10 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
   __shared__ uint32_t s_tile, s_pre, s_scan[2 * kFT / 32];
   WarpScan<kFT / 32> scan{s_scan, 0};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
+  // (no tile behind an error: the records of an automaton that failed to build mean nothing)
+  if (tid == 0) s_tile = *(volatile uint32_t *)err ? kNil : atomicAdd(tile_ctr, 1u);
   __syncthreads();
+  if (s_tile == kNil) return;
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * (kFT * I);
   const uint64_t seg = base + (uint64_t)warp * (I * 32) + lane;
@@ -1661,8 +1681,8 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
       Launch lp_(c, kKMarkEnds, P, s);
       k_rec_totals<<<grid_for(P, 256, sms), 256, 0, s>>>(rec, mtotal, P, misc + kMiscTraceCount, rtot);
     }
-    APO_TRY(seg_scan<false>(c, SrcU32{rtot}, DstExclusive{rtot, flat_off, misc + kMiscFlatTotal, P}, P, OpSum(),
-                            0u, s));
+    APO_TRY(seg_scan<false>(c, SrcU32{rtot}, DstExclusive{rtot, flat_off, misc + kMiscFlatTotal, P}, P,
+                            OpSatSum(), 0u, s));
     // read while the states are computed
     APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 1, misc + kMiscTraceCount, 4, cudaMemcpyDeviceToHost, s));
     APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscFlatTotal, 4, cudaMemcpyDeviceToHost, s));
@@ -1740,8 +1760,8 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   auto flatten = [&]() -> int {
     APO_TRY(ensure_side(c, flat_bytes, s));
     Launch lp_(c, kKAcFill, flat_total, s);
-    k_flat_chains<<<std::max(1, std::min(ceil_div(R, 8), sms * 16)), 256, 0, s>>>(rec, R, flat_off, ev,
-                                                                                  static_cast<uint32_t *>(c->side));
+    k_flat_chains<<<std::max(1, std::min(ceil_div(R, 8), sms * 16)), 256, 0, s>>>(
+        rec, R, flat_off, ev, P, static_cast<uint32_t *>(c->side), flat_total, c->ps.err);
     APO_CUDA_TRY(cudaGetLastError());
     return APO_OK;
   };
