@@ -756,13 +756,16 @@ struct OpSatSum {
   }
 };
 
-// One warp per record walks its chain and writes the ids.  Nothing is written
-// behind an error (the records and links of an automaton that failed to build
-// can point anywhere), nor past the P ids or the buffer's `entries`.
-__global__ void k_flat_chains(const uint4 *__restrict__ rec, uint32_t R, const uint32_t *__restrict__ flat_off,
+// One warp per record walks its chain and writes the ids, when their total
+// fits the buffer's `entries`.  Nothing is written behind an error (the
+// records and links of an automaton that failed to build can point anywhere),
+// nor past the P ids or the buffer.
+__global__ void k_flat_chains(const uint4 *__restrict__ rec, const uint32_t *__restrict__ R_dev,
+                              const uint32_t *__restrict__ flat_off, const uint32_t *__restrict__ total,
                               const uint32_t *__restrict__ evals, uint32_t P, uint32_t *__restrict__ flat,
                               uint64_t entries, uint32_t *err) {
-  if (*(volatile uint32_t *)err) return;
+  if (*(volatile uint32_t *)err || *total > entries) return;
+  const uint32_t R = min(P, *R_dev);
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += warps) {
@@ -1208,32 +1211,28 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
   }
   __syncthreads();
   uint32_t at = s_pre + ex;
-  if (sum == 0) return;  // (the whole warp)
+  if (sum == 0 || at >= cap) return;  // (the whole warp: no matches, or none that fits)
 #pragma unroll
   for (int i = 0; i < I; ++i) {
     const uint32_t inc = warp_inclusive(cnt[i], OpSum());
-    const uint32_t dst = at + inc - cnt[i], c0 = cnt[i];
+    const uint32_t dst = at + inc - cnt[i];
+    const uint32_t c0 = dst < cap ? (uint32_t)min((uint64_t)cnt[i], cap - dst) : 0u;  // of the chain, what fits
     at += __shfl_sync(0xffffffffu, inc, 31);
     const uint32_t src = c0 ? flat_off[rec[i]] : 0u;
     const uint32_t x = (uint32_t)(seg + i * 32);
     if (c0 <= kFillOwn) {  // short chains: each lane copies its own
       for (uint32_t k = 0; k < c0; ++k) {
-        if (dst + (uint64_t)k < cap) {
-          mend[dst + k] = x;
-          mid[dst + k] = flat[src + k];
-        }
+        mend[dst + k] = x;
+        mid[dst + k] = flat[src + k];
       }
     }
     for (uint32_t busy = __ballot_sync(0xffffffffu, c0 > kFillOwn); busy; busy &= busy - 1) {
       const int j = __ffs(busy) - 1;
       const uint32_t c = __shfl_sync(0xffffffffu, c0, j), sj = __shfl_sync(0xffffffffu, src, j);
-      const uint64_t dj = __shfl_sync(0xffffffffu, dst, j);
-      const uint32_t xj = __shfl_sync(0xffffffffu, x, j);
+      const uint32_t dj = __shfl_sync(0xffffffffu, dst, j), xj = __shfl_sync(0xffffffffu, x, j);
       for (uint32_t k = lane; k < c; k += 32) {
-        if (dj + k < cap) {
-          mend[dj + k] = xj;
-          mid[dj + k] = flat[sj + k];
-        }
+        mend[dj + k] = xj;
+        mid[dj + k] = flat[sj + k];
       }
     }
   }
@@ -1671,29 +1670,40 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   APO_CUDA_TRY(cudaGetLastError());
   if (n == 0) return check_device_error(c, s);  // synchronises
 
+  uint32_t *state = c->arena.take_n<uint32_t>(n);
+  uint32_t *off = c->arena.take_n<uint32_t>(n);  // flattened chains that fit it, or the positions' output offsets
+  if (!state || !off) return APO_ENOMEM;
   // record totals and flattened-chain offsets: they depend on the automaton
   // only, so they are queued now over the bound P >= records, and their
   // total is read with the match total below
   uint32_t *rtot = c->arena.take_n<uint32_t>(P), *flat_off = c->arena.take_n<uint32_t>(P);
   const bool flat_ok = rtot && flat_off;
+  const uint32_t *R_dev = misc + kMiscTraceCount, *flat_dev = misc + kMiscFlatTotal;
+  const int fblocks = std::max(1, std::min(ceil_div(P, 8), sms * 16));
   if (flat_ok) {
     {
       Launch lp_(c, kKMarkEnds, P, s);
-      k_rec_totals<<<grid_for(P, 256, sms), 256, 0, s>>>(rec, mtotal, P, misc + kMiscTraceCount, rtot);
+      k_rec_totals<<<grid_for(P, 256, sms), 256, 0, s>>>(rec, mtotal, P, R_dev, rtot);
     }
     APO_TRY(seg_scan<false>(c, SrcU32{rtot}, DstExclusive{rtot, flat_off, misc + kMiscFlatTotal, P}, P,
                             OpSatSum(), 0u, s));
     // read while the states are computed
-    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 1, misc + kMiscTraceCount, 4, cudaMemcpyDeviceToHost, s));
-    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscFlatTotal, 4, cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 1, flat_dev, 4, cudaMemcpyDeviceToHost, s));
     APO_CUDA_TRY(cudaEventRecord(c->round_ev[0], s));
+  }
+  // Each record's chain flattened once (their total is usually far below the
+  // match count).  Where the total is at most n, it goes to `off` now, and one
+  // kernel places and writes the matches; no more memory is taken before it is
+  // known that there is a match and room for it.  (Every pattern is in its own
+  // record's chain: more patterns than n never fit.)
+  const bool early = flat_ok && cap > 0 && P <= n;
+  if (early) {
+    Launch lp_(c, kKAcFill, P, s);
+    k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, off, n, c->ps.err);
   }
 
   // pass A: the state of every stream position (pass shape chosen above)
   Automaton A{nullptr, tsym, has_branch, g, skip, root, {skip}, (uint32_t)(maxlen / 32 + 2), {}};
-  uint32_t *state = c->arena.take_n<uint32_t>(n);
-  uint32_t *off = c->arena.take_n<uint32_t>(n);  // (offsets: only without flattened chains)
-  if (!state || !off) return APO_ENOMEM;
   if (halo) {
     // lifting tables of the skip links and of the preferred children
     uint32_t *hc = c->arena.take_n<uint32_t>((size_t)N + 1);
@@ -1742,41 +1752,32 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     APO_CUDA_TRY(cudaStreamSynchronize(s));
     if (c->host_pinned[0] == 0) break;
   }
-  // Flatten each output record's chain once (the sum over records of their
-  // chain lengths is usually far below the match count), then copy chains per
-  // position.  Very long flattened chains fall back to walking.
-  uint32_t R = 0;
   uint64_t flat_total = ~0ull;
   if (flat_ok) {
     APO_CUDA_TRY(cudaEventSynchronize(c->round_ev[0]));
-    R = c->host_pinned[1];
-    if (R) flat_total = c->host_pinned[2];
+    flat_total = c->host_pinned[1];
   }
-  const uint64_t flat_bytes = std::max<uint64_t>(flat_total, 1) * 4;
-  const bool flat = flat_total <= kMaxFlat;
-  // (with a caller workspace too small a side buffer is an error only once
-  // there is a match to write)
-  const bool fused = flat && !(c->ext && flat_bytes > c->side_bytes);
-  auto flatten = [&]() -> int {
-    APO_TRY(ensure_side(c, flat_bytes, s));
-    Launch lp_(c, kKAcFill, flat_total, s);
-    k_flat_chains<<<std::max(1, std::min(ceil_div(R, 8), sms * 16)), 256, 0, s>>>(
-        rec, R, flat_off, ev, P, static_cast<uint32_t *>(c->side), flat_total, c->ps.err);
-    APO_CUDA_TRY(cudaGetLastError());
+  // (with a caller workspace attached, chains longer than the side buffer are
+  // refused once there is a match to write)
+  const bool fused = early && flat_total <= n && !(c->ext && flat_total * 4 > c->side_bytes);
+  if (early) c->prof.adjust(kKAcFill, (flat_total <= n ? (int64_t)flat_total : 0) - (int64_t)P);
+  // the matches from flattened chains, or only their places; and their total
+  const bool wide = n >= (1ull << 22);
+  const int ftiles = ceil_div(n, kFT * (wide ? 8 : 2)), tiles = fused ? ftiles : ceil_div(n, kSTile);
+  auto fill = [&](const uint32_t *flat) -> int {
+    APO_TRY(ensure_lookback(c, ftiles));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
+    Launch lp_(c, kKAcFill, n, s);
+    (wide ? k_match_fill<8> : k_match_fill<2>)<<<ftiles, kFT, 0, s>>>(
+        state, (uint32_t)n, firstrec, rtot, flat_off, flat, match_end, match_id, cap, misc + kMiscCompactCount,
+        c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c), c->ps.err);
     return APO_OK;
   };
-  if (fused) APO_TRY(flatten());
-  // matches (or their offsets) and their total
-  const bool wide = n >= (1ull << 22);
-  const int tiles = fused ? ceil_div(n, kFT * (wide ? 8 : 2)) : ceil_div(n, kSTile);
-  APO_TRY(ensure_lookback(c, tiles));
-  APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
   if (fused) {
-    Launch lp_(c, kKAcFill, n, s);
-    (wide ? k_match_fill<8> : k_match_fill<2>)<<<tiles, kFT, 0, s>>>(
-        state, (uint32_t)n, firstrec, rtot, flat_off, static_cast<const uint32_t *>(c->side), match_end, match_id, cap,
-        misc + kMiscCompactCount, c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c), c->ps.err);
+    APO_TRY(fill(off));
   } else {
+    APO_TRY(ensure_lookback(c, tiles));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
     Launch lp_(c, kKMatchOffsets, n, s);
     k_match_offsets<<<tiles, kST, 0, s>>>(state, mtotal, (uint32_t)n, off, misc + kMiscCompactCount,
                                           c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c),
@@ -1795,8 +1796,15 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     return APO_ECAPACITY;
   }
   if (fused || !total_m) return APO_OK;  // synchronised above
-  if (flat) APO_TRY(flatten());  // (a caller workspace: no room, an error)
-  {
+  if (flat_total <= kMaxFlat) {  // longer chains, flattened beside the workspace
+    APO_TRY(ensure_side(c, flat_total * 4, s));
+    uint32_t *side = static_cast<uint32_t *>(c->side);
+    {
+      Launch lp_(c, kKAcFill, flat_total, s);
+      k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, side, flat_total, c->ps.err);
+    }
+    APO_TRY(fill(side));
+  } else {  // very long ones are walked
     Launch lp_(c, kKAcFill, n, s);
     k_ac_fill<<<grid_for(n, 256, sms), 256, 0, s>>>(state, (uint32_t)n, off, firstrec, rec, ev, match_end,
                                                     match_id, cap);

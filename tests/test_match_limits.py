@@ -1,7 +1,11 @@
-"""Matching at its limits: output chains whose flattened length passes 2^32."""
+"""Matching at its limits: output chains whose flattened length passes 2^32,
+chains longer than the stream, outputs with too little room."""
+import ctypes
+
 import numpy as np
 import pytest
 
+import oracle
 from test_gpu_parity import apo, tokens_dev  # noqa: F401 (apo: the fixture)
 
 pytestmark = pytest.mark.gpu
@@ -33,3 +37,62 @@ def test_chain_lengths_past_32_bits(apo):
     one = np.arange(copies, dtype=np.uint32)
     assert np.array_equal(as_u32(i), np.r_[one, one, np.uint32(copies), one])
     assert np.array_equal(as_u32(e), np.repeat(np.array([1, 4, 5], np.uint32), [copies, copies, copies + 1]))
+
+
+def raw_match(a, pats, off, stream, cap):
+    """(status, count, ends, ids) with one more entry than cap in both arrays."""
+    import torch
+    import paper_2406_18111_gb300 as gb
+    end = torch.full((cap + 1,), -1, dtype=torch.int32, device="cuda")
+    pid = torch.full((cap + 1,), -1, dtype=torch.int32, device="cuda")
+    count = ctypes.c_uint64()
+    p = gb.apo_patterns(len(off) - 1, pats.data_ptr(), 4, off.ctypes.data, None, None)
+    code = gb.lib().apo_match_candidates(a._h, ctypes.byref(p), stream.data_ptr(), stream.shape[0], end.data_ptr(),
+                                         pid.data_ptr(), cap, ctypes.byref(count), None)
+    torch.cuda.synchronize()
+    return code, int(count.value), end.cpu().numpy().view(np.uint32), pid.cpu().numpy().view(np.uint32)
+
+
+FLAT = 64 * 64 + 63 * 64 // 2  # entries of nested(64, 64)'s flattened chains
+
+
+@pytest.mark.parametrize("n", [50, FLAT - 1, FLAT, FLAT + 1, 3 * FLAT])
+def test_chains_around_the_stream_length(apo, n):
+    """Chains that fit beside the stream are flattened before the matches are
+    counted, longer ones after; with exactly the room, one entry less, none."""
+    import paper_2406_18111_gb300 as gb
+    pt, off = nested(64, 64)
+    text = np.full(n, 7, np.uint32)
+    text[::101] = 9
+    oe, oi = oracle.match(pt, off, text)
+    pats, stream = tokens_dev(pt, 4), tokens_dev(text, 4)
+    for cap in (len(oe), len(oe) - 1, 1000, 0):
+        code, count, e, i = raw_match(apo, pats, off, stream, cap)
+        assert count == len(oe) and e[cap] == i[cap] == 0xFFFFFFFF
+        assert code == (gb.APO_OK if cap == count else gb.APO_ECAPACITY)
+        if cap == count:
+            assert np.array_equal(e[:-1], oe) and np.array_equal(i[:-1], oi)
+
+
+def test_no_memory_for_chains_without_a_match():
+    """67.6 million entries of flattened chains (270 MB) and no match, or none
+    that fits: the context holds no more than for patterns of the same sizes
+    whose chains are short."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2406_18111_gb300 as gb
+    a = gb.Apo(0)
+    pt, off = nested(1 << 16, 1024)
+    flat, nest = tokens_dev(np.arange(len(pt)) + 100, 4), tokens_dev(pt, 4)
+    none, some = tokens_dev(np.full(4096, 9), 4), tokens_dev(np.full(4096, 7), 4)
+    assert raw_match(a, flat, off, none, 16)[:2] == (gb.APO_OK, 0)
+    raw_match(a, flat, off, none, 0)
+    free = torch.cuda.mem_get_info()[0]
+    assert raw_match(a, nest, off, none, 16)[:2] == (gb.APO_OK, 0)
+    assert raw_match(a, nest, off, none, 0)[:2] == (gb.APO_OK, 0)
+    want = (1 << 16) * 4096 + sum(min(x, 1023) for x in range(4096))
+    assert raw_match(a, nest, off, some, 16)[:2] == (gb.APO_ECAPACITY, want)
+    assert raw_match(a, nest, off, some, 0)[:2] == (gb.APO_ECAPACITY, want)
+    assert free - torch.cuda.mem_get_info()[0] < 32 << 20
+    a.close()
