@@ -362,7 +362,8 @@ int apo_finder_destroy(apo_finder *f);
  * Reports every (end, id) with stream[end - len(id) + 1 .. end] == pattern id,
  * for all patterns (overlapping occurrences included; a pattern listed twice
  * is reported under both ids), ordered by end ascending, then pattern length
- * descending, then id ascending.  At most 2^32 - 1 matches per call.
+ * descending, then id ascending.  At most 2^32 - 1 matches per call
+ * (APO_ECAPACITY beyond, whatever the capacity).
  * ---------------------------------------------------------------------- */
 typedef struct {
   uint64_t n_patterns;       /* P >= 1 */
@@ -392,7 +393,8 @@ typedef struct {
 /* Match `patterns` against stream[n] (device, same token width).  Writes the
  * matches to match_end/match_id (device, `cap` entries each) and their total
  * number to *count (HOST).  Synchronises `stream`.  APO_ECAPACITY if the total
- * exceeds cap (*count is exact, the arrays' contents are then unspecified).
+ * exceeds cap or 2^32 - 1 (*count is exact, the arrays' contents are then
+ * unspecified).
  * APO_EINVAL for an empty pattern, P = 0, or token_bytes not 4 or 8.
  * Performance only, the results are the same either way: when the slices are
  * taken from the stream itself (patterns->tokens == stream_tokens) and are

@@ -407,7 +407,7 @@ class Apo:
                              int(pat_tokens.shape[0]) if src_sa is not None else 0)
         code = lib().apo_match_candidates(self._h, ctypes.byref(p), _ptr(stream_tokens), n, _ptr(end),
                                           _ptr(pid), cap, ctypes.byref(cnt), _stream_handle(stream))
-        if code == APO_ECAPACITY:
+        if code == APO_ECAPACITY and cap < cnt.value < 1 << 32:
             return self.match_candidates(pat_tokens, pat_off, stream_tokens, int(cnt.value), stream,
                                          pat_start, pat_len, src_sa, src_lcp)
         _check(code)

@@ -1118,17 +1118,41 @@ __global__ void k_lift(const uint32_t *__restrict__ prev_a, uint32_t *__restrict
   }
 }
 
+// Adds the block's matches (v: the lane's) to *total.  64 bits: output places
+// are 32-bit sums, and when the total shows that those wrapped the call fails.
+// One addition per block; called by every warp, with a barrier between the two
+// halves.
+template <int NW>
+struct BlockTotal {
+  uint64_t *words;  // [NW] shared
+  __device__ __forceinline__ void put(uint64_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = v;
+  }
+  __device__ __forceinline__ void add(unsigned long long *total) {  // (by warp 1: warp 0 looks back)
+    if (threadIdx.x >> 5 != 1) return;
+    const uint32_t lane = threadIdx.x & 31;
+    uint64_t v = lane < NW ? words[lane] : 0ull;
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0 && v) atomicAdd(total, (unsigned long long)v);
+  }
+};
+
 // Exclusive prefix sum of total[state[x]] over stream positions (the first
 // output slot of each position), decoupled look-back.
 // A warp holds kSI rows of 32 consecutive positions (coalesced).
 constexpr int kST = 512, kSI = 8, kSTile = kST * kSI;
 __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restrict__ state,
                                                        const uint32_t *__restrict__ total, uint32_t n,
-                                                       uint32_t *__restrict__ off, uint32_t *sum_out,
+                                                       uint32_t *__restrict__ off, unsigned long long *matches,
                                                        uint64_t *status, uint32_t *tile_ctr,
                                                        uint32_t epoch, uint32_t *err) {
   __shared__ uint32_t s_tile, s_pre, s_scan[2 * kST / 32];
+  __shared__ uint64_t s_matches[kST / 32];
   WarpScan<kST / 32> scan{s_scan, 0};
+  BlockTotal<kST / 32> all{s_matches};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
   __syncthreads();
@@ -1136,6 +1160,7 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
   const uint64_t base = (uint64_t)t * kSTile;
   const uint64_t seg = base + (uint64_t)warp * (kSI * 32) + lane;
   uint32_t v[kSI], inc[kSI], sum = 0;
+  uint64_t mine = 0;
 #pragma unroll
   for (int i = 0; i < kSI; ++i) v[i] = seg + i * 32 < n ? state[seg + i * 32] : 0xffffffffu;
 #pragma unroll
@@ -1144,15 +1169,15 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
   for (int i = 0; i < kSI; ++i) {  // inclusive over the warp's positions
     inc[i] = sum + warp_inclusive(v[i], OpSum());
     sum = __shfl_sync(0xffffffffu, inc[i], 31);
+    mine += v[i];
   }
+  all.put(mine);
   uint32_t tot;
   const uint32_t ex = scan.run(sum, OpSum(), &tot);
+  all.add(matches);
   if (warp == 0) {
     const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
-    if (lane == 0) {
-      s_pre = pre;
-      if (base + kSTile >= n) *sum_out = pre + tot;
-    }
+    if (lane == 0) s_pre = pre;
   }
   __syncthreads();
   const uint32_t r = s_pre + ex;
@@ -1176,11 +1201,13 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
                                                     const uint32_t *__restrict__ rtot,
                                                     const uint32_t *__restrict__ flat_off,
                                                     const uint32_t *__restrict__ flat, uint32_t *__restrict__ mend,
-                                                    uint32_t *__restrict__ mid, uint64_t cap, uint32_t *sum_out,
-                                                    uint64_t *status, uint32_t *tile_ctr, uint32_t epoch,
-                                                    uint32_t *err) {
+                                                    uint32_t *__restrict__ mid, uint64_t cap,
+                                                    unsigned long long *matches, uint64_t *status,
+                                                    uint32_t *tile_ctr, uint32_t epoch, uint32_t *err) {
   __shared__ uint32_t s_tile, s_pre, s_scan[2 * kFT / 32];
+  __shared__ uint64_t s_matches[kFT / 32];
   WarpScan<kFT / 32> scan{s_scan, 0};
+  BlockTotal<kFT / 32> all{s_matches};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // (no tile behind an error: the records of an automaton that failed to build mean nothing)
   if (tid == 0) s_tile = *(volatile uint32_t *)err ? kNil : atomicAdd(tile_ctr, 1u);
@@ -1189,7 +1216,8 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
   const uint32_t t = s_tile;
   const uint64_t base = (uint64_t)t * (kFT * I);
   const uint64_t seg = base + (uint64_t)warp * (I * 32) + lane;
-  uint32_t rec[I], cnt[I], sum = 0;
+  uint32_t rec[I], cnt[I], sum;
+  uint64_t mine = 0;
 #pragma unroll
   for (int i = 0; i < I; ++i) rec[i] = seg + i * 32 < n ? state[seg + i * 32] : kNil;
 #pragma unroll
@@ -1197,17 +1225,16 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
 #pragma unroll
   for (int i = 0; i < I; ++i) {
     cnt[i] = rec[i] != kNil ? rtot[rec[i]] : 0u;
-    sum += cnt[i];
+    mine += cnt[i];
   }
-  sum = __reduce_add_sync(0xffffffffu, sum);
+  sum = __reduce_add_sync(0xffffffffu, (uint32_t)mine);
+  all.put(mine);
   uint32_t tot;
   const uint32_t ex = scan.run(sum, OpSum(), &tot);
+  all.add(matches);
   if (warp == 0) {
     const uint32_t pre = lb_sum_warp(status, t, tot, epoch, err);
-    if (lane == 0) {
-      s_pre = pre;
-      if (base + kFT * I >= n) *sum_out = pre + tot;
-    }
+    if (lane == 0) s_pre = pre;
   }
   __syncthreads();
   uint32_t at = s_pre + ex;
@@ -1762,37 +1789,39 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   const bool fused = early && flat_total <= n && !(c->ext && flat_total * 4 > c->side_bytes);
   if (early) c->prof.adjust(kKAcFill, (flat_total <= n ? (int64_t)flat_total : 0) - (int64_t)P);
   // the matches from flattened chains, or only their places; and their total
+  unsigned long long *matches = reinterpret_cast<unsigned long long *>(misc + kMiscMatchTotal);
   const bool wide = n >= (1ull << 22);
   const int ftiles = ceil_div(n, kFT * (wide ? 8 : 2)), tiles = fused ? ftiles : ceil_div(n, kSTile);
   auto fill = [&](const uint32_t *flat) -> int {
     APO_TRY(ensure_lookback(c, ftiles));
-    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchTiles, 0, 3 * sizeof(uint32_t), s));
     Launch lp_(c, kKAcFill, n, s);
     (wide ? k_match_fill<8> : k_match_fill<2>)<<<ftiles, kFT, 0, s>>>(
-        state, (uint32_t)n, firstrec, rtot, flat_off, flat, match_end, match_id, cap, misc + kMiscCompactCount,
-        c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c), c->ps.err);
+        state, (uint32_t)n, firstrec, rtot, flat_off, flat, match_end, match_id, cap, matches, c->ps.lookback,
+        misc + kMiscMatchTiles, next_epoch(c), c->ps.err);
     return APO_OK;
   };
   if (fused) {
     APO_TRY(fill(off));
   } else {
     APO_TRY(ensure_lookback(c, tiles));
-    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscCompactTiles, 0, 2 * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchTiles, 0, 3 * sizeof(uint32_t), s));
     Launch lp_(c, kKMatchOffsets, n, s);
-    k_match_offsets<<<tiles, kST, 0, s>>>(state, mtotal, (uint32_t)n, off, misc + kMiscCompactCount,
-                                          c->ps.lookback, misc + kMiscCompactTiles, next_epoch(c),
-                                          c->ps.err);
+    k_match_offsets<<<tiles, kST, 0, s>>>(state, mtotal, (uint32_t)n, off, matches, c->ps.lookback,
+                                          misc + kMiscMatchTiles, next_epoch(c), c->ps.err);
   }
   APO_CUDA_TRY(cudaGetLastError());
-  APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned, misc + kMiscCompactCount, 4, cudaMemcpyDeviceToHost, s));
+  APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned, matches, 8, cudaMemcpyDeviceToHost, s));
   APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + kPinnedErr, c->ps.err, sizeof(uint32_t),
                                cudaMemcpyDeviceToHost, s));
   APO_CUDA_TRY(cudaStreamSynchronize(s));
   APO_TRY(device_error_status(c, s));
-  const uint64_t total_m = c->host_pinned[0];
+  uint64_t total_m;
+  memcpy(&total_m, c->host_pinned, 8);
   *count = total_m;
-  if (total_m > cap) {
-    set_error("match_candidates: more matches than cap (count written)");
+  if (total_m > cap || total_m > 0xffffffffull) {
+    set_error(total_m > cap ? "match_candidates: more matches than cap (count written)"
+                            : "match_candidates: more than 2^32 - 1 matches (count written)");
     return APO_ECAPACITY;
   }
   if (fused || !total_m) return APO_OK;  // synchronised above

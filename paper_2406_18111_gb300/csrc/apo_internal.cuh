@@ -68,7 +68,7 @@ enum : int {
 };
 enum : int {
   kMiscRefreshTiles = 0, kMiscRefreshCount, kMiscCompactTiles, kMiscCompactCount,
-  kMiscCandCount, kMiscMaxLen, kMiscAccCount, kMiscTraceCount, kMiscMatchCount,
+  kMiscCandCount, kMiscMaxLen, kMiscAccCount, kMiscTraceCount,
   kMiscKeyOr = 16,        // two u64 (four words): OR and maximum of keys
   kMiscRound = 20,        // two words: active-suffix counts of consecutive doubling rounds
   kMiscDict = 22,         // two words: distinct tokens, dictionary overflow flag
@@ -80,6 +80,8 @@ enum : int {
   kMiscRoundW = 32,       // 2 x 4 words of consecutive doubling rounds (see build_suffix_array)
   kMiscSmall = 48,        // 8 words of a small-window call (see small.cu)
   kMiscDictHits = 56,     // tokens the dictionary held already when they came
+  kMiscMatchTiles = 57,   // tile tickets of the match output
+  kMiscMatchTotal = 58,   // matches (u64), behind their tickets
   kMiscCount = 64,
 };
 

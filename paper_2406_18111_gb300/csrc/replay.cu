@@ -863,6 +863,7 @@ int replay_stream(apo_ctx *c, const void *tokens, uint64_t n, int tb, const apo_
     Carve cv2{static_cast<char *>(c->rp[2])};
     v = carve2(cv2, cap);
     const int r = match_patterns(c, &pp, tokens, n, v.oend, v.oid, cap, &O, s, w.sp, w.slcp);
+    if (r == APO_ECAPACITY && O >= 0x7fffffffull) break;  // (refused below)
     if (r == APO_ECAPACITY && attempt == 0) {
       cap = O;
       continue;

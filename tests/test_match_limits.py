@@ -1,5 +1,6 @@
 """Matching at its limits: output chains whose flattened length passes 2^32,
-chains longer than the stream, outputs with too little room."""
+chains longer than the stream, outputs with too little room, more matches
+than 32 bits hold."""
 import ctypes
 
 import numpy as np
@@ -96,3 +97,24 @@ def test_no_memory_for_chains_without_a_match():
     assert raw_match(a, nest, off, some, 0)[:2] == (gb.APO_ECAPACITY, want)
     assert free - torch.cuda.mem_get_info()[0] < 32 << 20
     a.close()
+
+
+@pytest.mark.parametrize("copies,n", [(1 << 20, 4096), (4097, 1 << 20), (4097, 1 << 22)])
+def test_more_matches_than_32_bits(apo, copies, n):
+    """The count is exact past 2^32 (it was taken modulo 2^32: 0, 2^20 and 2^22
+    here), with the chains flattened after the count and before it."""
+    import paper_2406_18111_gb300 as gb
+    pt, off = nested(copies, 1)
+    assert copies * n >= 1 << 32
+    code, count, e, i = raw_match(apo, tokens_dev(pt, 4), off, tokens_dev(np.full(n, 7), 4), 1 << 23)
+    assert (code, count) == (gb.APO_ECAPACITY, copies * n)
+    assert e[-1] == i[-1] == 0xFFFFFFFF
+
+
+def test_replay_refuses_more_occurrences_than_31_bits(apo):
+    """2^20 tokens and the slices 7 .. 7^4200: 4.4e9 occurrences."""
+    from paper_2406_18111_gb300 import ApoError
+    n, q = 1 << 20, 4200
+    start, length = tokens_dev(np.zeros(q), 4), tokens_dev(np.arange(1, q + 1), 4)
+    with pytest.raises(ApoError, match="APO_EINVAL.*occurrences"):
+        apo.replay(tokens_dev(np.full(n, 7), 4), start, length, start)
