@@ -119,7 +119,18 @@ uint64_t key_hash(const std::vector<uint32_t> &win, const std::vector<const void
   return h;
 }
 
+// One window's offsets are {0, its counts}: a capture stages them for several
+// windows only.
 void write_offsets(const GraphEntry &e, uint32_t W, apo_repeats_out *out) {
+  if (W == 1) {
+    uint64_t *const dst[3] = {out->cand_off, out->sel_off, out->trace_off};
+    for (int k = 0; k < 3; ++k)
+      if (dst[k]) {
+        dst[k][0] = 0;
+        dst[k][1] = e.counts[k];
+      }
+    return;
+  }
   for (uint32_t w = 0; w <= W; ++w) {
     if (out->cand_off) out->cand_off[w] = e.stage[w];
     if (out->sel_off) out->sel_off[w] = e.stage[(W + 1) + w];
@@ -224,6 +235,7 @@ int graph_batched(apo_ctx *c, const apo_windows *ws, const apo_repeats_params *p
             cudaMallocHost(&e.bad_host, 4) == cudaSuccess;
   if (ok && !rec.vals.empty())
     ok = cudaMemcpy(e.dev_vals, rec.vals.data(), rec.vals.size() * 4, cudaMemcpyHostToDevice) == cudaSuccess;
+  if (ok) memset(e.stage, 0, 3 * (size_t)(W + 1) * 4);  // (a call without candidates copies nothing to it)
   if (!ok) {  // no graph; the recorded call's results stand
     cudaGetLastError();
     free_entry(e);
