@@ -83,3 +83,88 @@ def test_capacities_and_missing_outputs(apo):
         assert counts[:3].tolist() == [len(want.cand_len), len(want.sel_start), len(want.trace_len)]
         got = sel.cpu().numpy().view(np.uint32)
         assert np.array_equal(got[:cap], want.sel_start[:cap]) and (got[cap:] == 0xFFFFFFFF).all()
+
+
+@pytest.mark.parametrize("tb", [4, 8])
+@pytest.mark.parametrize("lens", [(8192,) * 3, (700, 0, 5000, 1, 64), tuple(i % 3 for i in range(12000)), (1,)])
+def test_caller_workspace(apo, lens, tb):
+    """A caller workspace of exactly the queried size holds the small windows'
+    scratch, for many tiny windows as well; a byte less is refused."""
+    import torch
+    from paper_2406_18111_gb300 import Apo, ApoError
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    t = tokens_dev(window("loop", int(off[-1]), 8).astype(np.uint64) * np.uint64(2654435761 if tb == 4 else 1 << 33), tb)
+    want = apo.find_repeats_batched(t, off, 2)
+    a = Apo(0)
+    need = a.find_repeats_workspace(off)
+    buf = torch.empty(need, dtype=torch.uint8, device="cuda")
+    a.set_workspace(buf)
+    a.profile_reset()
+    for _ in range(2):
+        got = a.find_repeats_batched(t, off, 2)
+        for f in FIELDS + ("cand_accepted",):
+            assert bool((getattr(got, f) == getattr(want, f)).all()), f
+        for f in ("cand_off", "sel_off", "trace_off"):
+            assert np.array_equal(getattr(got, f), getattr(want, f)), f
+    assert a.profile_read()["small"][0] == 2
+    a.set_workspace(buf[:need - 1])
+    with pytest.raises(ApoError, match="APO_ENOMEM"):
+        a.find_repeats_batched(t, off, 2)
+    a.set_workspace(None)
+    a.close()
+
+
+def rounds_of(S, lcp, windows=1):
+    """The doubling rounds reported: the first key holds h0 tokens (as plain
+    values, or dense codes where fewer than four of those fit), and round r runs
+    iff some LCP is at least h0 * 2^(r-1)."""
+    S = np.asarray(S, np.uint64)
+    top = int(S.max())
+    bits = (windows - 1).bit_length() if windows > 1 else 0
+    h0 = (64 - bits) // (top + 1).bit_length() if top < 1 << 32 else 0
+    if h0 < 4 and len(S) >= 4096:
+        sigma = len(np.unique(S[S != np.uint64(2**64 - 1)]))
+        cap = min(1 << (2 * len(S) - 1).bit_length(), 1 << 23)
+        if sigma <= cap // 2:
+            h0 = max(h0, (64 - bits) // (sigma + 1).bit_length())
+    h0 = min(h0, 32) if h0 >= 2 else 1
+    r = 0
+    while int(lcp.max()) >= h0 << r:
+        r += 1
+    return r
+
+
+@pytest.mark.parametrize("kind,tb", [("loop", 4), ("run", 4), ("random", 4), ("random", 8), ("few", 4), ("tasks", 8)])
+@pytest.mark.parametrize("n", [1, 64, 1000, 4095, 4096, 8192, 8193, 1 << 15])
+def test_rounds_reported(apo, kind, tb, n):
+    """The same count from both paths (here and just past 8,192 tokens)."""
+    from paper_2406_18111_gb300 import as_u32
+    S = window(kind, n, 70 + n)
+    r = apo.find_repeats(tokens_dev(S, tb), 5)
+    assert r.rounds == rounds_of(S, as_u32(r.lcp))
+
+
+@pytest.mark.parametrize("tb", [4, 8])
+@pytest.mark.parametrize("lens", [(1300000,), ((1 << 21) + (1 << 14),), (700000, 0, 9000, 1, 600000)])
+def test_mostly_distinct_windows(apo, lens, tb):
+    """Millions of nearly distinct tokens: where a first key would hold two of
+    them (the last two shapes) it holds one, with the window in a batch; the
+    rounds reported stay those of two."""
+    from paper_2406_18111_gb300 import as_u32
+    n = sum(lens)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    S = W.splitmix64(11, n) >> np.uint64(34)  # 30-bit values
+    S[500:800] = S[100:400]
+    S[9500:11000] = S[15000:16500]
+    S[n - 3000:n - 2000] = 5  # a run
+    r = apo.find_repeats_batched(tokens_dev(S, tb), off, 5)
+    assert r.rounds == rounds_of(S, as_u32(r.lcp), len(lens)) > 5
+    for w in range(len(lens)):
+        a, b = int(off[w]), int(off[w + 1])
+        if b - a < 2:
+            continue
+        o = oracle.find_repeats(S[a:b], 5, sa_method="doubling")
+        assert np.array_equal(as_u32(r.sa)[a:b], o.sa) and np.array_equal(as_u32(r.lcp)[a:b], o.lcp)
+        s0, s1, t0, t1 = (int(x) for x in (r.sel_off[w], r.sel_off[w + 1], r.trace_off[w], r.trace_off[w + 1]))
+        assert np.array_equal(as_u32(r.sel_start)[s0:s1], o.sel_start)
+        assert np.array_equal(as_u32(r.trace_len)[t0:t1], o.trace_len)
