@@ -111,26 +111,28 @@ struct Dict {
   uint64_t mask;
 };
 
-// Four tokens per thread, whose first slots' reads are under way together.
+// kI tokens per thread, whose first slots' reads are under way together (one
+// up to kDictOne tokens per SM: 290,000 distinct ones 14 us, with four 24).
 // Lanes that find the same slot empty leave the insertion to the first of
 // them: the tokens of a task stream are few, and the first reads of the whole
 // chip see them missing.
 constexpr int kDictI = 4;
-template <class T>
+constexpr uint32_t kDictOne = 2048;
+template <class T, int kI>
 __global__ void k_dict_insert(const T *__restrict__ tok, uint64_t m, Dict d) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kDictI;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kI;
   const uint32_t lt = lanemask_lt();
-  for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kDictI; b0 < m; b0 += stride) {
-    uint64_t t[kDictI], cur[kDictI];
+  for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kI; b0 < m; b0 += stride) {
+    uint64_t t[kI], cur[kI];
 #pragma unroll
-    for (int u = 0; u < kDictI; ++u) {  // (all-ones: mapped to a reserved symbol instead)
+    for (int u = 0; u < kI; ++u) {  // (all-ones: mapped to a reserved symbol instead)
       const uint64_t i = b0 + (uint64_t)u * blockDim.x + threadIdx.x;
       t[u] = i < m ? (uint64_t)tok[i] : kEmpty;
     }
 #pragma unroll
-    for (int u = 0; u < kDictI; ++u) cur[u] = t[u] != kEmpty ? d.keys[mix64(t[u]) & d.mask] : kEmpty;
+    for (int u = 0; u < kI; ++u) cur[u] = t[u] != kEmpty ? d.keys[mix64(t[u]) & d.mask] : kEmpty;
 #pragma unroll
-    for (int u = 0; u < kDictI; ++u) {
+    for (int u = 0; u < kI; ++u) {
       uint64_t slot = mix64(t[u]) & d.mask;
       const bool need = t[u] != kEmpty && cur[u] == kEmpty;
       if (__any_sync(0xffffffffu, need)) {
@@ -185,7 +187,10 @@ __global__ void k_dict_map(const T *__restrict__ tok, uint64_t m, Dict d, uint32
       const uint64_t i = i0 + (uint64_t)u * blockDim.x;
       if (i >= m) continue;
       const uint64_t slot = mix64(t[u]) & d.mask;
-      sym[i] = t[u] != kEmpty && cur[u] == t[u] ? (uint32_t)slot : dict_symbol(d, (T)t[u]);
+      if (t[u] != kEmpty && (cur[u] == t[u] || cur[u] == kEmpty))  // settled at the first slot
+        sym[i] = cur[u] == t[u] ? (uint32_t)slot : kNil;
+      else
+        sym[i] = dict_symbol(d, (T)t[u]);
     }
   }
 }
@@ -1494,12 +1499,14 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   APO_TRY(seg_scan<false>(c, SrcPlen{plen}, DstTstart{plen, tstart}, P, OpSum(), 0u, s));
   {
     Launch lp_(c, kKDictInsert, extent, s);
+    const bool few = extent <= (uint64_t)sms * kDictOne;
+    const int blocks = grid_for(few ? extent : (extent + kDictI - 1) / kDictI, 256, sms);
     if (tb == 4)
-      k_dict_insert<<<grid_for((extent + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint32_t *>(pp->tokens),
-                                                                extent, d);
+      (few ? k_dict_insert<uint32_t, 1> : k_dict_insert<uint32_t, kDictI>)<<<blocks, 256, 0, s>>>(
+          static_cast<const uint32_t *>(pp->tokens), extent, d);
     else
-      k_dict_insert<<<grid_for((extent + kDictI - 1) / kDictI, 256, sms), 256, 0, s>>>(static_cast<const uint64_t *>(pp->tokens),
-                                                                extent, d);
+      (few ? k_dict_insert<uint64_t, 1> : k_dict_insert<uint64_t, kDictI>)<<<blocks, 256, 0, s>>>(
+          static_cast<const uint64_t *>(pp->tokens), extent, d);
   }
   {
     Launch lp_(c, kKPatLayout, N, s);

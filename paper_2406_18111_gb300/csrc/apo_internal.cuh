@@ -71,7 +71,6 @@ enum : int {
   kMiscCandCount, kMiscMaxLen, kMiscAccCount, kMiscTraceCount,
   kMiscKeyOr = 16,        // two u64 (four words): OR and maximum of keys
   kMiscRound = 20,        // two words: active-suffix counts of consecutive doubling rounds
-  kMiscDict = 22,         // two words: distinct tokens, dictionary overflow flag
   kMiscPhaseLen = 24,     // two words: list lengths of consecutive greedy phases
   kMiscFixChanged = 26,   // two words: changes of consecutive automaton repair passes
   kMiscFlatTotal = 28,    // length of the flattened output chains
@@ -79,9 +78,9 @@ enum : int {
   kMiscRoundTiles = 30,   // tile tickets of a doubling round
   kMiscRoundW = 32,       // 2 x 4 words of consecutive doubling rounds (see build_suffix_array)
   kMiscSmall = 48,        // 8 words of a small-window call (see small.cu)
-  kMiscDictHits = 56,     // tokens the dictionary held already when they came
   kMiscMatchTiles = 57,   // tile tickets of the match output
   kMiscMatchTotal = 58,   // matches (u64), behind their tickets
+  kMiscDict = 60,         // three words: distinct tokens, dictionary overflow flag, tokens held already when they came
   kMiscCount = 64,
 };
 

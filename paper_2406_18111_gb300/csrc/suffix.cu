@@ -310,13 +310,18 @@ __device__ __forceinline__ uint64_t token_at(const void *tokens, int tb, uint32_
 // past `limit` of them.  A warp adds its new tokens to the count at once:
 // with one addition per new token, 2^22 of them (a window of random tokens,
 // where the dictionary is given up) queued on one address for 0.8 ms.
+// kI tokens per thread: their first slots' reads are under way together.  One
+// where every token can have a thread of its own: four in a row are a longer
+// chain (the dictionary's kernels over random tokens, one / four per thread:
+// 80,000 38 / 49 us, 200,000 55 / 61, 311,000 73 / 69).
+constexpr uint32_t kDictOne = 1536;  // tokens per SM up to which it is one
+template <int kI>
 __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t n, uint64_t *keys, uint64_t mask,
                               uint32_t limit, uint32_t *distinct, uint32_t *over, uint32_t *hits) {
   __shared__ uint32_t s_hits;  // tokens found present, of those looked at before the dictionary was given up
   if (threadIdx.x == 0) s_hits = 0;
   __syncthreads();
   uint32_t held = 0;
-  constexpr int kI = 4;  // tokens per thread: their first slots' reads are under way together
   const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kI;
   for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kI; b0 < n; b0 += stride) {
@@ -1199,8 +1204,8 @@ uint64_t dict_capacity(uint32_t n) {
 
 // Order-preserving dense codes of the tokens (1 .. sigma, sigma + 1 for the
 // all-ones u64 token) through a dictionary of the distinct tokens.  begin
-// queues the inserts and the read-back of the distinct count and overflow
-// flag (pinned words 2 and 3); finish, after the caller's synchronisation,
+// queues the inserts and the read-back of the distinct count, overflow flag
+// and hits (pinned words 2 to 4); finish, after the caller's synchronisation,
 // leaves *codes_out null when there are more than half the dictionary's
 // capacity of distinct tokens.
 struct DictCodes {
@@ -1226,18 +1231,15 @@ int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCod
   if (!d->ok) return APO_OK;
   uint32_t *misc = c->ps.counters + kCtrMisc;
   APO_CUDA_TRY(cudaMemsetAsync(d->keys, 0xff, d->cap * sizeof(uint64_t), s));
-  APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDict, 0, 2 * sizeof(uint32_t), s));
-  APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDictHits, 0, sizeof(uint32_t), s));
+  APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscDict, 0, 3 * sizeof(uint32_t), s));
   {
     Launch lp_(c, kKSaDict, n, s);
-    k_dict_tokens<<<grid_for((n + 3) / 4, 256, c->num_sms), 256, 0, s>>>(tokens, tb, n, d->keys, d->cap - 1, limit,
-                                                               misc + kMiscDict, misc + kMiscDict + 1,
-                                                               misc + kMiscDictHits);
+    const bool few = n <= (uint32_t)c->num_sms * kDictOne;
+    (few ? k_dict_tokens<1> : k_dict_tokens<4>)<<<grid_for(few ? n : (n + 3) / 4, 256, c->num_sms), 256, 0, s>>>(
+        tokens, tb, n, d->keys, d->cap - 1, limit, misc + kMiscDict, misc + kMiscDict + 1, misc + kMiscDict + 2);
   }
-  if (!capturing(c)) {  // read in dictionary_finish (a captured call takes it from its tape there)
-    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscDict, 8, cudaMemcpyDeviceToHost, s));
-    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 4, misc + kMiscDictHits, 4, cudaMemcpyDeviceToHost, s));
-  }
+  if (!capturing(c))  // read in dictionary_finish (a captured call takes it from its tape there)
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscDict, 12, cudaMemcpyDeviceToHost, s));
   return APO_OK;
 }
 
