@@ -1198,7 +1198,12 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
 // reads and writes).  Offsets written and read back cost two more passes over
 // the positions (2^26 of them: 315 us for the offsets, 341 for the copy).
 // I: rows per warp; fewer on short streams, for more tiles.
+// A warp's rows are 32 I consecutive positions: where the matches of a long
+// stream lie on a few of them (256 positions with 4,096 each), the copies of
+// one warp set the time (1.2 ms of 1.9).  Rows of more than kHeavyRow matches
+// are listed instead, and k_match_heavy copies them, a block per row.
 constexpr uint32_t kFillOwn = 4;
+constexpr uint32_t kHeavyRow = 4096;
 constexpr int kFT = 512;
 template <int I>
 __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__ state, uint32_t n,
@@ -1207,7 +1212,8 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
                                                     const uint32_t *__restrict__ flat_off,
                                                     const uint32_t *__restrict__ flat, uint32_t *__restrict__ mend,
                                                     uint32_t *__restrict__ mid, uint64_t cap,
-                                                    unsigned long long *matches, uint64_t *status,
+                                                    unsigned long long *matches, uint2 *__restrict__ heavy,
+                                                    uint32_t *heavy_n, uint64_t *status,
                                                     uint32_t *tile_ctr, uint32_t epoch, uint32_t *err) {
   __shared__ uint32_t s_tile, s_pre, s_scan[2 * kFT / 32];
   __shared__ uint64_t s_matches[kFT / 32];
@@ -1247,9 +1253,14 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
 #pragma unroll
   for (int i = 0; i < I; ++i) {
     const uint32_t inc = warp_inclusive(cnt[i], OpSum());
-    const uint32_t dst = at + inc - cnt[i];
+    const uint32_t dst = at + inc - cnt[i], all_row = __shfl_sync(0xffffffffu, inc, 31);
+    if (all_row > kHeavyRow) {
+      if (lane == 0) heavy[atomicAdd(heavy_n, 1u)] = make_uint2((uint32_t)((seg + i * 32) >> 5), at);
+      at += all_row;
+      continue;
+    }
     const uint32_t c0 = dst < cap ? (uint32_t)min((uint64_t)cnt[i], cap - dst) : 0u;  // of the chain, what fits
-    at += __shfl_sync(0xffffffffu, inc, 31);
+    at += all_row;
     const uint32_t src = c0 ? flat_off[rec[i]] : 0u;
     const uint32_t x = (uint32_t)(seg + i * 32);
     if (c0 <= kFillOwn) {  // short chains: each lane copies its own
@@ -1264,6 +1275,33 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
       const uint32_t dj = __shfl_sync(0xffffffffu, dst, j), xj = __shfl_sync(0xffffffffu, x, j);
       for (uint32_t k = lane; k < c; k += 32) {
         mend[dj + k] = xj;
+        mid[dj + k] = flat[sj + k];
+      }
+    }
+  }
+}
+
+// The rows of 32 positions that k_match_fill listed (row, its first output
+// place), when all matches fit: a block per row copies chain after chain.
+__global__ void __launch_bounds__(256) k_match_heavy(const uint2 *__restrict__ heavy, uint32_t rows,
+                                                     const uint32_t *__restrict__ state, uint32_t n,
+                                                     const uint32_t *__restrict__ firstrec,
+                                                     const uint32_t *__restrict__ rtot,
+                                                     const uint32_t *__restrict__ flat_off,
+                                                     const uint32_t *__restrict__ flat, uint32_t *__restrict__ mend,
+                                                     uint32_t *__restrict__ mid) {
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t h = blockIdx.x; h < rows; h += gridDim.x) {
+    const uint2 row = heavy[h];
+    const uint64_t x = (uint64_t)row.x * 32 + lane;
+    const uint32_t r = x < n ? firstrec[state[x]] : kNil;
+    const uint32_t cnt = r != kNil ? rtot[r] : 0u, src = r != kNil ? flat_off[r] : 0u;
+    const uint32_t dst = row.y + warp_inclusive(cnt, OpSum()) - cnt;
+    for (int j = 0; j < 32; ++j) {  // (every warp holds the row)
+      const uint32_t c = __shfl_sync(0xffffffffu, cnt, j), sj = __shfl_sync(0xffffffffu, src, j);
+      const uint32_t dj = __shfl_sync(0xffffffffu, dst, j);
+      for (uint32_t k = threadIdx.x; k < c; k += blockDim.x) {
+        mend[dj + k] = row.x * 32 + j;
         mid[dj + k] = flat[sj + k];
       }
     }
@@ -1494,7 +1532,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
 
   // symbols: the dictionary of pattern tokens, the pattern text, the stream
   APO_CUDA_TRY(cudaMemsetAsync(d.keys, 0xff, dct * sizeof(uint64_t), s));
-  uint32_t *ssym = c->arena.take_n<uint32_t>(std::max<uint64_t>(n, 1));
+  uint32_t *ssym = c->arena.take_n<uint32_t>(std::max<uint64_t>(n, 2));  // (later: the heavy rows' list)
   if (!ssym) return APO_ENOMEM;
   APO_TRY(seg_scan<false>(c, SrcPlen{plen}, DstTstart{plen, tstart}, P, OpSum(), 0u, s));
   {
@@ -1799,39 +1837,57 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   unsigned long long *matches = reinterpret_cast<unsigned long long *>(misc + kMiscMatchTotal);
   const bool wide = n >= (1ull << 22);
   const int ftiles = ceil_div(n, kFT * (wide ? 8 : 2)), tiles = fused ? ftiles : ceil_div(n, kSTile);
+  uint2 *heavy = reinterpret_cast<uint2 *>(ssym);  // (8 bytes per 32 positions; the symbols are used up)
   auto fill = [&](const uint32_t *flat) -> int {
     APO_TRY(ensure_lookback(c, ftiles));
-    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchTiles, 0, 3 * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchHeavy, 0, 4 * sizeof(uint32_t), s));
     Launch lp_(c, kKAcFill, n, s);
     (wide ? k_match_fill<8> : k_match_fill<2>)<<<ftiles, kFT, 0, s>>>(
-        state, (uint32_t)n, firstrec, rtot, flat_off, flat, match_end, match_id, cap, matches, c->ps.lookback,
-        misc + kMiscMatchTiles, next_epoch(c), c->ps.err);
+        state, (uint32_t)n, firstrec, rtot, flat_off, flat, match_end, match_id, cap, matches, heavy,
+        misc + kMiscMatchHeavy, c->ps.lookback, misc + kMiscMatchTiles, next_epoch(c), c->ps.err);
     return APO_OK;
   };
   if (fused) {
     APO_TRY(fill(off));
   } else {
     APO_TRY(ensure_lookback(c, tiles));
-    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchTiles, 0, 3 * sizeof(uint32_t), s));
+    APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscMatchHeavy, 0, 4 * sizeof(uint32_t), s));
     Launch lp_(c, kKMatchOffsets, n, s);
     k_match_offsets<<<tiles, kST, 0, s>>>(state, mtotal, (uint32_t)n, off, matches, c->ps.lookback,
                                           misc + kMiscMatchTiles, next_epoch(c), c->ps.err);
   }
-  APO_CUDA_TRY(cudaGetLastError());
-  APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned, matches, 8, cudaMemcpyDeviceToHost, s));
-  APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + kPinnedErr, c->ps.err, sizeof(uint32_t),
-                               cudaMemcpyDeviceToHost, s));
-  APO_CUDA_TRY(cudaStreamSynchronize(s));
-  APO_TRY(device_error_status(c, s));
+  // the output's words and the error word
+  auto read_out = [&]() -> int {
+    APO_CUDA_TRY(cudaGetLastError());
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned, misc + kMiscMatchHeavy, 16, cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + kPinnedErr, c->ps.err, sizeof(uint32_t),
+                                 cudaMemcpyDeviceToHost, s));
+    APO_CUDA_TRY(cudaStreamSynchronize(s));
+    return device_error_status(c, s);
+  };
+  // the rows that the fill left
+  auto fill_heavy = [&](const uint32_t *flat) -> int {
+    const uint32_t rows = c->host_pinned[0];
+    if (!rows) return APO_OK;
+    {
+      Launch lp_(c, kKAcFill, rows, s);
+      k_match_heavy<<<std::min<uint32_t>(rows, sms * 8), 256, 0, s>>>(heavy, rows, state, (uint32_t)n, firstrec, rtot,
+                                                                      flat_off, flat, match_end, match_id);
+    }
+    APO_CUDA_TRY(cudaGetLastError());
+    return check_device_error(c, s);  // synchronises
+  };
+  APO_TRY(read_out());
   uint64_t total_m;
-  memcpy(&total_m, c->host_pinned, 8);
+  memcpy(&total_m, c->host_pinned + 2, 8);
   *count = total_m;
   if (total_m > cap || total_m > 0xffffffffull) {
     set_error(total_m > cap ? "match_candidates: more matches than cap (count written)"
                             : "match_candidates: more than 2^32 - 1 matches (count written)");
     return APO_ECAPACITY;
   }
-  if (fused || !total_m) return APO_OK;  // synchronised above
+  if (!total_m) return APO_OK;  // synchronised above
+  if (fused) return fill_heavy(off);
   if (flat_total <= kMaxFlat) {  // longer chains, flattened beside the workspace
     APO_TRY(ensure_side(c, flat_total * 4, s));
     uint32_t *side = static_cast<uint32_t *>(c->side);
@@ -1840,6 +1896,8 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
       k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, side, flat_total, c->ps.err);
     }
     APO_TRY(fill(side));
+    APO_TRY(read_out());
+    return fill_heavy(side);
   } else {  // very long ones are walked
     Launch lp_(c, kKAcFill, n, s);
     k_ac_fill<<<grid_for(n, 256, sms), 256, 0, s>>>(state, (uint32_t)n, off, firstrec, rec, ev, match_end,

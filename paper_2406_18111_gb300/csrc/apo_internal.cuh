@@ -78,8 +78,9 @@ enum : int {
   kMiscRoundTiles = 30,   // tile tickets of a doubling round
   kMiscRoundW = 32,       // 2 x 4 words of consecutive doubling rounds (see build_suffix_array)
   kMiscSmall = 48,        // 8 words of a small-window call (see small.cu)
-  kMiscMatchTiles = 57,   // tile tickets of the match output
-  kMiscMatchTotal = 58,   // matches (u64), behind their tickets
+  kMiscMatchHeavy = 56,   // the match output's words: rows left to a second kernel,
+  kMiscMatchTiles = 57,   // tile tickets
+  kMiscMatchTotal = 58,   // and matches (u64)
   kMiscDict = 60,         // three words: distinct tokens, dictionary overflow flag, tokens held already when they came
   kMiscCount = 64,
 };

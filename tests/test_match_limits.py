@@ -1,6 +1,6 @@
 """Matching at its limits: output chains whose flattened length passes 2^32,
 chains longer than the stream, outputs with too little room, more matches
-than 32 bits hold."""
+than 32 bits hold, matches on few positions."""
 import ctypes
 
 import numpy as np
@@ -118,3 +118,24 @@ def test_replay_refuses_more_occurrences_than_31_bits(apo):
     start, length = tokens_dev(np.zeros(q), 4), tokens_dev(np.arange(1, q + 1), 4)
     with pytest.raises(ApoError, match="APO_EINVAL.*occurrences"):
         apo.replay(tokens_dev(np.full(n, 7), 4), start, length, start)
+
+
+@pytest.mark.parametrize("n,start,k,copies", [(1, 0, 1, 4097), (40, 7, 33, 4096), (5000, 1000, 32, 128),
+                                              (5000, 1024, 32, 128), (5000, 1024, 32, 129), (5000, 1010, 32, 300),
+                                              (20001, 19993, 8, 9000), ((1 << 22) + 5, 4096, 256, 1000),
+                                              ((1 << 22) + 5, (1 << 22) - 90, 95, 500)])
+def test_matches_on_few_positions(apo, n, start, k, copies):
+    """k positions with `copies` matches each: rows of 32 positions at and past
+    4,096 matches, cut by the stream's end, in both tile shapes."""
+    import paper_2406_18111_gb300 as gb
+    pt, off = nested(copies, 1)
+    text = np.full(n, 9, np.uint32)
+    text[start:start + k] = 7
+    m = k * copies
+    for cap in (m, m - 1):
+        code, count, e, i = raw_match(apo, tokens_dev(pt, 4), off, tokens_dev(text, 4), cap)
+        assert (code, count) == (gb.APO_OK if cap == m else gb.APO_ECAPACITY, m)
+        assert e[cap] == i[cap] == 0xFFFFFFFF
+        if cap == m:
+            assert np.array_equal(e[:m], np.repeat(np.arange(start, start + k, dtype=np.uint32), copies))
+            assert np.array_equal(i[:m], np.tile(np.arange(copies, dtype=np.uint32), k))
