@@ -225,6 +225,7 @@ uint64_t interval_sets(int n, int m) {
 int optimum_batched(apo_ctx *c, const apo_windows *ws, uint32_t min_len, uint32_t *best, uint32_t *wstart,
                     uint32_t *wlen, uint32_t *wcount, cudaStream_t s) {
   const uint64_t W = ws->n_windows;
+  min_len = std::min<uint32_t>(min_len, kOptMax + 1);  // longer than any window: no traces
   uint64_t maxn = 0;
   for (uint64_t w = 0; w < W; ++w) maxn = std::max(maxn, ws->win_off[w + 1] - ws->win_off[w]);
   if (maxn > (uint64_t)kOptMax) {
