@@ -384,7 +384,7 @@ int find_repeats_from_sa(apo_ctx *c, const void *tokens, int token_bytes, const 
 
 // Small windows (small.cu): whether a call's windows all take that path, and
 // the call (the workspace is reserved; results and counts as in apo.h).
-bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest);
+bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest, int token_bytes);
 int small_find_repeats(apo_ctx *c, const void *tokens, int token_bytes, const uint64_t *win_off, uint32_t windows,
                        uint32_t longest, const apo_repeats_params *p, apo_repeats_out *out, cudaStream_t s);
 int small_init();

@@ -444,7 +444,7 @@ int find_repeats_driver(apo_ctx *c, const void *tokens, int tb, uint64_t total,
   }
   uint64_t longest = 0;
   for (uint32_t w = 0; w < nwin; ++w) longest = std::max(longest, win_off[w + 1] - win_off[w]);
-  if (small_windows(c->num_sms, n, nwin, longest))
+  if (small_windows(c->num_sms, n, nwin, longest, tb))
     return small_find_repeats(c, tokens, tb, win_off, nwin, (uint32_t)longest, p, out, s);
   SuffixState st;
   st.n = n;

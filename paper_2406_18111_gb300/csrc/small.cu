@@ -913,22 +913,35 @@ int read_words(apo_ctx *c, const uint32_t *dev, uint32_t *host, int words, cudaS
 
 }  // namespace
 
-// Whether a call's windows go through k_small: each at most 8,192 tokens (what
-// fits a block's shared memory), and not so many that the general path, which
-// shares its launches among any number of windows, is the faster one.  Both
-// sides' times are modelled from measurements (152 SMs; u32 loops with noise):
-// a block of 1,024 threads holds an SM for about 22 us + 30 ns per token, one
-// of 256 threads (windows of up to 512 tokens; eight are resident) for 10 us +
-// 24 ns per token, and as windows learn their output places in order, the
-// longest one sets the pace; the general path takes about 850 us + 0.45 ns
-// per token.  Measured (here / general path, us): 1 x 512 57 / 443, 1 x 4,096
-// 144 / 576, 1 x 8,192 266 / 687, 300 x 8,192 549 / 1,789, 2,000 x 600 564 /
-// 1,172, 10,000 x 128 855 / 1,190; past the line: 20,000 x 64 1,457 / 1,188,
-// 4,000 of 64 to 2,000 tokens 1,599 / 1,399.
-bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest) {
+// Whether a call's windows go through k_small: each at most 8,192 tokens (what fits a
+// block's shared memory), and not so many that the general path, which shares its
+// launches among any number of windows, is the faster one.  Both sides' times are
+// modelled from measurements (152 SMs), on the contents that favour the general path
+// most -- four tokens at random, whose groups are gone after a few rounds -- so that
+// hardly a call is slower here than there: a block of 1,024 threads holds an SM for
+// about 24 us + 25 ns per token of the longest window, one of 256 threads (windows of
+// up to 512 tokens; eight are resident) for 10.3 us + 18.5 ns, u32 tokens 15% less;
+// the general path takes about 750 us + 0.24 ns per token, a little more per token of
+// longer windows.  Windows below 64 tokens, with fewer rounds, cost both sides less:
+// 8.5 us + 47 ns per token here, 450 us + 4.7 us per token there.
+// Measured (here / general path, us), u64 tokens, loops with noise and four tokens at
+// random: 10,000 x 64 933 / 1,010 and 834 / 887; 5,000 x 513 1,607 / 1,929 and 1,340 /
+// 1,381; 5,000 x 600 1,671 / 2,051 and 1,395 / 1,486; 10,000 x 1,000 3,862 / 4,751 and
+// 3,237 / 3,305; 3,000 x 8,192 5,486 / 10,639 and 4,538 / 9,156; past the line: 12,000
+// x 8 678 / 554 and 758 / 522; 20,000 x 128 2,038 / 1,794 and 1,709 / 1,360; 50,000 x
+// 250 5,706 / 5,537 and 4,553 / 3,634; 10,000 x 600 3,196 / 3,232 and 2,669 / 2,226;
+// 50,000 x 513 14,510 / 10,626 and 11,994 / 6,883.
+// What the line costs: loops up to 1.13 times (20,000 x 1,000 u64), random u64 tokens
+// up to 1.7 times.
+bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest, int token_bytes) {
   if (longest > kSmall[kSmallShapes - 1].max_n) return false;
-  const double block = longest <= kSmall[0].max_n ? 10.0 + 0.024 * (double)longest : 22.0 + 0.030 * (double)longest;
-  return (double)windows * block / sms < 850.0 + 0.00045 * (double)total;
+  const double len = (double)longest;
+  const double block = longest > kSmall[0].max_n ? 24.0 + 0.0252 * len
+                       : longest >= 64           ? 10.3 + 0.0185 * len
+                                                 : 8.5 + 0.047 * len;
+  const double general = longest >= 64 ? 750.0 : 450.0 + 4.7 * len;
+  return (double)windows * block * (token_bytes == 4 ? 0.85 : 1.0) / sms <
+         general + (0.00024 + 1.3e-8 * len) * (double)total;
 }
 
 int small_init() {

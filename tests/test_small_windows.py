@@ -86,7 +86,7 @@ def test_capacities_and_missing_outputs(apo):
 
 
 @pytest.mark.parametrize("tb", [4, 8])
-@pytest.mark.parametrize("lens", [(8192,) * 3, (700, 0, 5000, 1, 64), tuple(i % 3 for i in range(12000)), (1,)])
+@pytest.mark.parametrize("lens", [(8192,) * 3, (700, 0, 5000, 1, 64), tuple(i % 3 for i in range(6000)), (1,)])
 def test_caller_workspace(apo, lens, tb):
     """A caller workspace of exactly the queried size holds the small windows'
     scratch, for many tiny windows as well; a byte less is refused."""
@@ -168,3 +168,28 @@ def test_mostly_distinct_windows(apo, lens, tb):
         s0, s1, t0, t1 = (int(x) for x in (r.sel_off[w], r.sel_off[w + 1], r.trace_off[w], r.trace_off[w + 1]))
         assert np.array_equal(as_u32(r.sel_start)[s0:s1], o.sel_start)
         assert np.array_equal(as_u32(r.trace_len)[t0:t1], o.trace_len)
+
+
+@pytest.mark.parametrize("windows,n,tb,small", [(10000, 600, 8, False), (50000, 250, 8, False), (20000, 128, 4, False),
+                                                (12000, 2, 8, False), (6000, 2, 8, True),
+                                                (5000, 600, 8, True), (10000, 64, 8, True), (300, 8192, 4, True)])
+def test_many_windows_take_the_faster_path(apo, windows, n, tb, small):
+    """Thousands of short windows go the general path where its shared launches
+    are the faster ones; the results are those of smaller batches, which go
+    window by window."""
+    t = tokens_dev(window("few", windows * n, 3), tb)
+    off = np.arange(windows + 1, dtype=np.uint64) * np.uint64(n)
+    apo.profile_reset()
+    r = apo.find_repeats_batched(t, off, 5, stages=False)
+    assert ("small" in apo.profile_read()) == small
+    at, step = 0, 1250
+    for w in range(0, windows, step):
+        k = min(step, windows - w)
+        apo.profile_reset()
+        p = apo.find_repeats_batched(t[w * n:(w + k) * n], off[:k + 1], 5, stages=False)
+        assert "small" in apo.profile_read()
+        for f, o in (("sel_start", "sel_off"), ("sel_len", "sel_off"), ("sel_trace", "sel_off"),
+                     ("trace_len", "trace_off"), ("trace_start", "trace_off")):
+            ro, po = getattr(r, o), getattr(p, o)
+            assert np.array_equal(ro[w:w + k + 1] - ro[w], po), o
+            assert bool((getattr(r, f)[int(ro[w]):int(ro[w + k])] == getattr(p, f)).all()), f
