@@ -48,6 +48,7 @@
 // going is finished in O(levels) steps by binary lifting over the level
 // ranks; finally LCP[k] = PLCP[SA[k+1]] (LCP[k] pairs SA[k] with SA[k+1]).
 #include <algorithm>
+#include <numeric>
 #include <cstring>
 
 #include "apo_internal.cuh"
@@ -315,16 +316,20 @@ __device__ __forceinline__ uint64_t token_at(const void *tokens, int tb, uint32_
 // chain (the dictionary's kernels over random tokens, one / four per thread:
 // 80,000 38 / 49 us, 200,000 55 / 61, 311,000 73 / 69).
 constexpr uint32_t kDictOne = 1536;  // tokens per SM up to which it is one
+// The blocks' tokens are visited `step` apart (modulo their number, to which
+// it is coprime), so that what has been seen when the dictionary is given up
+// stands for the whole window.
 template <int kI>
 __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t n, uint64_t *keys, uint64_t mask,
-                              uint32_t limit, uint32_t *distinct, uint32_t *over, uint32_t *hits) {
+                              uint32_t limit, uint32_t step, uint32_t *distinct, uint32_t *over, uint32_t *hits) {
   __shared__ uint32_t s_hits;  // tokens found present, of those looked at before the dictionary was given up
   if (threadIdx.x == 0) s_hits = 0;
   __syncthreads();
   uint32_t held = 0;
   const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * kI;
-  for (uint64_t b0 = (uint64_t)blockIdx.x * blockDim.x * kI; b0 < n; b0 += stride) {
+  const uint32_t chunk = blockDim.x * kI, chunks = (n + chunk - 1) / chunk;
+  for (uint32_t q = blockIdx.x; q < chunks; q += gridDim.x) {
+    const uint64_t b0 = (uint64_t)q * step % chunks * chunk;
     if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) break;
     uint64_t t[kI], cur[kI];
     uint32_t fresh = 0;
@@ -1214,7 +1219,7 @@ struct DictCodes {
   uint32_t *slot_code = nullptr, *codes = nullptr;
   SortBuffers lb;
   bool ok = false;
-  bool mostly_distinct = false;  // fewer than one token in nine had come before
+  bool mostly_distinct = false;  // fewer than one token in three had come before
 };
 
 int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCodes *d, cudaStream_t s) {
@@ -1235,8 +1240,13 @@ int dictionary_begin(apo_ctx *c, const void *tokens, int tb, uint32_t n, DictCod
   {
     Launch lp_(c, kKSaDict, n, s);
     const bool few = n <= (uint32_t)c->num_sms * kDictOne;
+    uint32_t step = 1;  // (all tokens are seen when their number cannot pass the limit)
+    if (n > limit) {
+      const uint32_t chunks = (uint32_t)ceil_div(n, 256 * 4);
+      for (step = chunks / 8 * 5 + 1; std::gcd(step, chunks) != 1;) ++step;
+    }
     (few ? k_dict_tokens<1> : k_dict_tokens<4>)<<<grid_for(few ? n : (n + 3) / 4, 256, c->num_sms), 256, 0, s>>>(
-        tokens, tb, n, d->keys, d->cap - 1, limit, misc + kMiscDict, misc + kMiscDict + 1, misc + kMiscDict + 2);
+        tokens, tb, n, d->keys, d->cap - 1, limit, step, misc + kMiscDict, misc + kMiscDict + 1, misc + kMiscDict + 2);
   }
   if (!capturing(c))  // read in dictionary_finish (a captured call takes it from its tape there)
     APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 2, misc + kMiscDict, 12, cudaMemcpyDeviceToHost, s));
@@ -1260,7 +1270,7 @@ int dictionary_finish(apo_ctx *c, const void *tokens, int tb, uint32_t n, int tb
   } else {
     sv[0] = c->host_pinned[2];
     sv[1] = c->host_pinned[3];
-    few = (uint64_t)c->host_pinned[4] * 8 < sv[0];
+    few = (uint64_t)c->host_pinned[4] * 2 < sv[0];
     if (recording(c)) {
       tape_put(c, sv, 2);
       tape_put(c, &few, 1);
@@ -1403,6 +1413,10 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
   // (2^24 random u32 tokens: four passes instead of eight), and a round over
   // the few that are left.  Level L then stands for 2^L tokens instead of
   // 2^(L+1); the rounds reported stay those of the two-token key, one fewer.
+  // One token / two, 2^24 u32 tokens with a looping share: none 2.64 / 3.54 ms,
+  // 5% 5.50 / 6.23, 20% 9.88 / 10.4, 35% (about the line) 14.2 / 14.4, 50% 18.5
+  // / 18.5, 75% 25.9 / 25.5; 2^22 u64: none 1.83 / 1.99, 35% 5.63 / 5.60, 50%
+  // 6.77 / 6.68.
   const bool one = h0 == 2 && dict.mostly_distinct;
   if (one) h0 = 1;
   // level 0: groups of equal first h0 tokens (within a window)

@@ -193,3 +193,18 @@ def test_many_windows_take_the_faster_path(apo, windows, n, tb, small):
             ro, po = getattr(r, o), getattr(p, o)
             assert np.array_equal(ro[w:w + k + 1] - ro[w], po), o
             assert bool((getattr(r, f)[int(ro[w]):int(ro[w + k])] == getattr(p, f)).all()), f
+
+
+@pytest.mark.parametrize("distinct,loops", [(14 << 20, 2 << 20), (12 << 20, 12 << 20)])
+def test_key_length_does_not_depend_on_the_order(apo, distinct, loops):
+    """Three times as many distinct tokens as the dictionary takes (2^22), and
+    loops before, behind or between them: the same first key, which shows in the
+    rounds run."""
+    a = W.splitmix64(5, distinct) >> np.uint64(33)
+    b = W.periodic_window(loops, 50, 0.05, 1000, 6).astype(np.uint64)
+    seen = set()
+    for S in (np.r_[a, b], np.r_[b, a], np.r_[a[:distinct // 2], b, a[distinct // 2:]]):
+        apo.profile_reset()
+        r = apo.find_repeats(tokens_dev(S, 4), 5, stages=False)
+        seen.add((apo.profile_read()["minor"][0], r.rounds))
+    assert len(seen) == 1, seen
