@@ -62,7 +62,7 @@ struct Arena {
 enum : int {
   kCtrSortHist = 0,       // radix sort digit histograms, 12 places x 512 digits
   kCtrSortTiles = 6144,   // radix sort tile tickets, 12
-  kCtrSortBuf = 6160,     // which buffer holds the pairs before each place of a sort that may skip places, 13
+  kCtrSortMoved = 6160,   // places that moved the pairs before each place of a sort that may skip places, 12
   kCtrMisc = 6208,        // per-kernel tile tickets and totals, see kMisc*
   kCtrWords = 8192,
 };
@@ -322,10 +322,10 @@ uint32_t *sort_first_hist(apo_ctx *c);
 int radix_sort_planned(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &sp, cudaStream_t s,
                        const uint32_t *n_dev, bool hist_ready);
 // The same from b's buffer 0 for keys that may agree in whole digits: a place
-// where they do moves nothing, and the buffer that holds the result is known
-// on the device only (*buf: 0 or 1).
+// where they do moves nothing.  The device word *moved (zero on entry) gets the
+// places that moved; buffer *moved & 1 holds the result.
 int radix_sort_skipping(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &sp, cudaStream_t s,
-                        const uint32_t *n_dev, const uint32_t **buf);
+                        const uint32_t *n_dev, uint32_t *moved);
 // OR of all keys (how many digits are populated) in out_dev[0] and their
 // maximum in out_dev[1]; both words must be zero on entry.
 void launch_key_or(apo_ctx *c, const uint64_t *keys, uint32_t n, uint64_t *out_dev, cudaStream_t s);

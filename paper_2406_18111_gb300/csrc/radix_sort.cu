@@ -35,8 +35,8 @@ namespace {
 constexpr int kHistThreads = 256;
 constexpr int kMaxRadix = 512;
 constexpr int kMaxPass = 12;
-constexpr int kCtrSortEnd = kCtrSortBuf + kMaxPass + 1;  // the sort's counters from kCtrSortHist on
-static_assert(kCtrSortHist == 0 && kCtrSortTiles == kMaxPass * kMaxRadix && kCtrSortTiles + kMaxPass <= kCtrSortBuf &&
+constexpr int kCtrSortEnd = kCtrSortMoved + kMaxPass;  // the sort's counters from kCtrSortHist on
+static_assert(kCtrSortHist == 0 && kCtrSortTiles == kMaxPass * kMaxRadix && kCtrSortTiles + kMaxPass <= kCtrSortMoved &&
                   kCtrSortEnd <= kCtrMisc,
               "the sort's counters are cleared in one piece");
 
@@ -136,19 +136,20 @@ __global__ void __launch_bounds__(TPB, (KO ? 1536 : 1024) / TPB) k_rs_pass(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint64_t *__restrict__ kout,
     uint32_t *__restrict__ vout, uint32_t n, const uint32_t *__restrict__ n_dev, int place,
     const uint32_t *__restrict__ gcnt, int next_place, uint32_t *__restrict__ next_cnt, uint64_t *status,
-    uint32_t *tile_ctr, uint32_t epoch, uint32_t *err, uint32_t *buf) {
+    uint32_t *tile_ctr, uint32_t epoch, uint32_t *err, const uint32_t *moved, uint32_t *moved_out) {
   using S = PassShape<TPB, ITEMS, BITS, KO>;
   if (n_dev) n = min(n, *n_dev);  // the launch is sized for an upper bound
   constexpr int R = S::kRadix, NW = S::kWarps, TILE = S::kTile;
   if (SKIP) {
     // A sort that may skip places (an instantiation of its own: the others
-    // lose 4% to the two reads ahead of everything else): *buf says which buffer holds the pairs
-    // before this one.  When every key has the same digit there is nothing to
-    // move; only the next place's digits are counted.
-    const uint32_t f = *buf;
+    // lose 4% to the two reads ahead of everything else): *moved places before
+    // this one moved the pairs, which says which buffer holds them.  When
+    // every key has the same digit there is nothing to move; only the next
+    // place's digits are counted.
+    const uint32_t f = *moved;
     const int same = __syncthreads_or(threadIdx.x < R && gcnt[threadIdx.x] == n);
-    if (blockIdx.x == 0 && threadIdx.x == 0) buf[1] = same ? f : f ^ 1u;
-    if (f) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *moved_out = same ? f : f + 1;
+    if (f & 1u) {
       const uint64_t *ki = kin;
       kin = kout;
       kout = const_cast<uint64_t *>(ki);
@@ -342,7 +343,7 @@ __global__ void k_rs_trial_keys(uint64_t *keys, uint32_t *vals, uint32_t n, int 
 // ---------------------------------------------------------------- shapes
 using PassFn = void (*)(const uint64_t *, const uint32_t *, uint64_t *, uint32_t *, uint32_t, const uint32_t *,
                         int, const uint32_t *, int, uint32_t *, uint64_t *, uint32_t *, uint32_t, uint32_t *,
-                        uint32_t *);
+                        const uint32_t *, uint32_t *);
 using HistFn = void (*)(const uint64_t *, const uint32_t *, uint32_t, const uint32_t *, int, uint32_t *);
 
 struct Shape {
@@ -378,13 +379,14 @@ int plan(const Shape &sh, const DigitRange *ranges, int nranges, Places *pl) {
 
 // All passes of one sort with one shape (b.cur flips once per pass).
 int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uint32_t *n_dev, const Places &pl,
-              bool count, cudaStream_t s, bool hist_ready = false, uint32_t *buf = nullptr) {
+              bool count, cudaStream_t s, bool hist_ready = false, uint32_t *moved = nullptr) {
   const int R = 1 << sh.bits;
   const int tile = sh.threads * sh.items;
   const int tiles = ceil_div(n, tile);
   APO_TRY(ensure_lookback(c, (size_t)tiles * R));
   uint32_t *hist = c->ps.counters + kCtrSortHist;   // [kMaxPass][kMaxRadix]
   uint32_t *tctr = c->ps.counters + kCtrSortTiles;  // [kMaxPass]
+  uint32_t *before = c->ps.counters + kCtrSortMoved;  // [kMaxPass] (a sort that may skip places)
   if (hist_ready) {  // the first place's counts are in; clear the others and the tile tickets
     APO_CUDA_TRY(cudaMemsetAsync(hist + kMaxRadix, 0, (kCtrSortEnd - kMaxRadix) * sizeof(uint32_t), s));
   } else {
@@ -399,13 +401,13 @@ int sort_with(apo_ctx *c, const Shape &sh, SortBuffers &b, uint32_t n, const uin
     {
       const bool ko = b.vals[b.cur] == nullptr;
       Launch lp_(c, count ? (ko ? kKRsPassKeys : kKRsPass) : kKRsTune, n, s);
-      (ko ? sh.pass_keys : sh.pass)[buf != nullptr]<<<tiles, sh.threads, ko ? sh.smem_keys : sh.smem, s>>>(
+      (ko ? sh.pass_keys : sh.pass)[moved != nullptr]<<<tiles, sh.threads, ko ? sh.smem_keys : sh.smem, s>>>(
           b.keys[b.cur], b.vals[b.cur], b.keys[b.cur ^ 1],
                                                  b.vals[b.cur ^ 1], n, n_dev, pl.p[p], hist + p * kMaxRadix, nxt,
                                                  hist + (p + 1) * kMaxRadix, c->ps.lookback, tctr + p, ep,
-                                                 c->ps.err, buf ? buf + p : nullptr);
+                                                 c->ps.err, before + p, p + 1 < pl.n ? before + p + 1 : moved);
     }
-    if (!buf) b.cur ^= 1;
+    if (!moved) b.cur ^= 1;
   }
   APO_CUDA_TRY(cudaGetLastError());
   return APO_OK;
@@ -570,18 +572,13 @@ int radix_sort_planned(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &s
 }
 
 int radix_sort_skipping(apo_ctx *c, SortBuffers &b, uint32_t n, const SortPlan &sp, cudaStream_t s,
-                        const uint32_t *n_dev, const uint32_t **buf) {
-  uint32_t *w = c->ps.counters + kCtrSortBuf;
-  *buf = w + std::max(0, sp.places);
+                        const uint32_t *n_dev, uint32_t *moved) {
   b.cur = 0;
-  if (sp.shape < 0) {  // nothing to sort: buffer 0
-    *buf = nullptr;
-    return APO_OK;
-  }
+  if (sp.shape < 0) return APO_OK;  // nothing to sort
   Places pl;
   pl.n = sp.places;
   for (int p = 0; p < sp.places; ++p) pl.p[p] = sp.place[p];
-  return sort_with(c, kShapes[sp.shape], b, n, n_dev, pl, true, s, true, w);
+  return sort_with(c, kShapes[sp.shape], b, n, n_dev, pl, true, s, true, moved);
 }
 
 int radix_sort_pairs(apo_ctx *c, SortBuffers &b, uint32_t n, const DigitRange *ranges, int nranges,

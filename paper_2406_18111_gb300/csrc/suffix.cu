@@ -159,9 +159,9 @@ __global__ void __launch_bounds__(kST) k_split(
     int finals, uint32_t *__restrict__ snap, uint32_t *__restrict__ sa, uint32_t *__restrict__ rank,
     uint8_t *__restrict__ fin, uint32_t *__restrict__ nid, uint32_t *__restrict__ nhd, uint32_t list_cap,
     uint32_t *count_out, uint32_t n, uint64_t *st_max, uint64_t *st_sum, uint32_t *tile_ctr, uint32_t epoch,
-    uint32_t *err, int id_bits, const uint64_t *keys1, const uint32_t *vals1, const uint32_t *buf) {
+    uint32_t *err, int id_bits, const uint64_t *keys1, const uint32_t *vals1, const uint32_t *moved) {
   constexpr int NW = kST / 32;
-  if (buf && *buf) {  // the sort left its result in the other buffer
+  if (moved && (*moved & 1u)) {  // the sort left its result in the other buffer
     keys = keys1;
     vals = vals1;
   }
@@ -1180,7 +1180,7 @@ int split_launch(apo_ctx *c, bool big, const uint64_t *keys, const uint32_t *val
                  const uint32_t *bg_pos, uint32_t bg_cap, uint32_t level, bool finals, uint32_t *snap,
                  SuffixState &st, uint32_t *nid, uint32_t *nhd, uint32_t *count_out, cudaStream_t s,
                  int id_bits = 0, const uint64_t *keys1 = nullptr, const uint32_t *vals1 = nullptr,
-                 const uint32_t *buf = nullptr) {
+                 const uint32_t *moved = nullptr) {
   const int tiles = std::max(1, ceil_div(ub, kSTile));
   APO_TRY(ensure_lookback(c, (size_t)2 * tiles));
   uint32_t *misc = c->ps.counters + kCtrMisc;
@@ -1191,7 +1191,7 @@ int split_launch(apo_ctx *c, bool big, const uint64_t *keys, const uint32_t *val
     k_split<true><<<tiles, kST, 0, s>>>(keys, vals, ub, n_dev, ord_shift, bg_head, bg_off, bg_pos, bg_cap, level,
                                         finals, snap, st.sa, st.rank, st.fin, nid, nhd, st.n, count_out, st.n,
                                         c->ps.lookback, c->ps.lookback + tiles, misc + kMiscRefreshTiles, ep,
-                                        c->ps.err, id_bits, keys1, vals1, buf);
+                                        c->ps.err, id_bits, keys1, vals1, moved);
   else
     k_split<false><<<tiles, kST, 0, s>>>(keys, vals, ub, n_dev, 0, nullptr, nullptr, nullptr, 0, level, finals,
                                          snap, st.sa, st.rank, st.fin, nid, nhd, st.n, count_out, st.n,
@@ -1467,7 +1467,7 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
   // the holed list (hid, hhd) and writes the big entries' keys; the big
   // entries are sorted and k_split settles them into the holed list; then
   // k_list_compact drops the holes.  The round's device words (next list
-  // length, big entries, -, big groups) alternate between two slots.  The host queues round r + 1 before it has read round r's
+  // length, big entries, places that moved them, big groups) alternate between two slots.  The host queues round r + 1 before it has read round r's
   // length (an upper bound sizes the launches), and stops one round after
   // the length reaches 0 (that round's kernels find nothing to do).  A round
   // with no big entries has no big groups after it, so from then on the big
@@ -1489,11 +1489,11 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
     const int64_t d = (int64_t)len - (int64_t)rb[rr].ub;
     for (int id : {(int)kKMinor, (int)kKRound, (int)kKListCompact}) c->prof.adjust(id, d);
   };
-  auto exact_big = [&](uint32_t rr, uint32_t cnt) {  // round rr had cnt big entries
+  auto exact_big = [&](uint32_t rr, uint32_t cnt, uint32_t moved) {  // round rr had cnt big entries, moved so many times
     if (!rb[rr].places) return;
-    const int64_t d = (int64_t)cnt - (int64_t)rb[rr].big_ub;
-    c->prof.adjust(rb[rr].keys ? kKRsPassKeys : kKRsPass, d * rb[rr].places);
-    c->prof.adjust(kKSplit, d);
+    c->prof.adjust(rb[rr].keys ? kKRsPassKeys : kKRsPass,
+                   (int64_t)cnt * moved - (int64_t)rb[rr].big_ub * rb[rr].places);
+    c->prof.adjust(kKSplit, (int64_t)cnt - (int64_t)rb[rr].big_ub);
   };
   for (uint32_t r = 1;; ++r) {
     if (st.levels >= max_levels) {
@@ -1580,10 +1580,9 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
       if (id_bits) bb.vals[0] = bb.vals[1] = nullptr;
       // the ordinals' bits are sized for as many big groups as the entries
       // could form; with few and large ones (runs) whole digits are zero
-      const uint32_t *buf = nullptr;
-      APO_TRY(radix_sort_skipping(c, bb, big_ub, sp, s, words + 1, &buf));
+      APO_TRY(radix_sort_skipping(c, bb, big_ub, sp, s, words + 1, words + 2));
       APO_TRY(split_launch(c, true, bb.keys[0], bb.vals[0], big_ub, words + 1, mb, bg_head, bg_off, bg_pos, bg_cap,
-                           r, true, st.snaps[r], st, hid, hhd, nullptr, s, id_bits, bb.keys[1], bb.vals[1], buf));
+                           r, true, st.snaps[r], st, hid, hhd, nullptr, s, id_bits, bb.keys[1], bb.vals[1], words + 2));
     }
     APO_CUDA_TRY(cudaMemsetAsync(misc + kMiscRoundTiles, 0, sizeof(uint32_t), s));
     {
@@ -1596,7 +1595,7 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
     const bool cap = capturing(c);
     if (!cap) {
       if (r == 1) APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 6, first_count, 4, cudaMemcpyDeviceToHost, s));
-      APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 16 + 2 * (r & 1), words, 8, cudaMemcpyDeviceToHost, s));
+      APO_CUDA_TRY(cudaMemcpyAsync(c->host_pinned + 16 + 4 * (r & 1), words, 12, cudaMemcpyDeviceToHost, s));
       APO_CUDA_TRY(cudaEventRecord(c->round_ev[r & 1], s));
     }
     if (r == 1) continue;
@@ -1615,28 +1614,30 @@ int build_suffix_array(apo_ctx *c, const void *tokens, int tb, uint32_t n, Suffi
       if (first == 0) {  // the first sort left no group: rounds 1 and 2 idle
         if (!cap) {
           exact_list(2, 0);
-          exact_big(1, 0);
-          exact_big(2, 0);
+          exact_big(1, 0, 0);
+          exact_big(2, 0, 0);
         }
         st.levels = 1;
         break;
       }
     }
-    uint32_t w2[2];
+    uint32_t w2[2], moved = 0;
     if (cap) {
       APO_TRY(tape_take(c, misc + kMiscRoundW + 4 * ((r - 1) & 1), w2, 2, s));
     } else {
       if (r > 2) APO_CUDA_TRY(cudaEventSynchronize(c->round_ev[(r - 1) & 1]));
-      w2[0] = c->host_pinned[16 + 2 * ((r - 1) & 1)];
-      w2[1] = c->host_pinned[17 + 2 * ((r - 1) & 1)];
+      const uint32_t *p = c->host_pinned + 16 + 4 * ((r - 1) & 1);
+      w2[0] = p[0];
+      w2[1] = p[1];
+      moved = p[2];
       if (recording(c)) tape_put(c, w2, 2);
     }
     if (!cap) {
       exact_list(r, w2[0]);
-      exact_big(r - 1, w2[1]);
+      exact_big(r - 1, w2[1], moved);
     }
     if (w2[0] == 0) {  // round r had nothing to do: levels 0 .. r - 1
-      if (!cap) exact_big(r, 0);
+      if (!cap) exact_big(r, 0, 0);
       st.levels = (int)r;
       break;
     }
