@@ -684,6 +684,9 @@ __global__ void __launch_bounds__(TPB, 1) k_small(const SmallArgs a) {
     // ---- greedy: rounds of growing size; survivors (ends unmarked) settled
     // 32 at a time by warp 0, as in k_greedy
     const uint64_t smask = (1ull << nb) - 1;
+    // the lists lie over the codes, suffixes and ranks, which are used up (not
+    // over lcp, which the accepted starts take over below)
+    static_assert(3 * TPB * sizeof(uint32_t) <= (NMAX + 64 + 2 * NMAX) * sizeof(uint16_t), "the greedy's lists end before lcp");
     uint32_t *list = reinterpret_cast<uint32_t *>(code);  // [TPB] survivors: (start << 16) | end
     uint32_t *lk = list + TPB;                             // [TPB] their candidates
     uint32_t *lov = lk + TPB;                              // [TPB] overlap masks
