@@ -97,7 +97,7 @@ struct Persistent {
 // ---------------------------------------------------------------- instrumentation
 enum KernelId : int {
   kKHash, kKInitKeys, kKKeyOr, kKRsHist, kKRsOffsets, kKRsPass, kKRefresh, kKPack, kKPhi,
-  kKPlcp, kKLcpPerm, kKMin32, kKMax, kKCandGen, kKCompact, kKCandGather, kKGreedy, kKTraces,
+  kKPlcp, kKLcpPerm, kKMin32, kKMax, kKCandGen, kKCompact, kKGreedy, kKTraces,
   kKSelOut, kKPatLayout, kKTableInit, kKEndPairs, kKMarkEnds, kKAcFix, kKAcStates,
   kKAcFill, kKDictInsert, kKDictMap, kKSlices, kKMatchOffsets, kKSegScan, kKStarts, kKSparse,
   kKAcNodes, kKAcJump, kKRsTune, kKRpPieces, kKRpNeed, kKRpChain, kKRpAppear, kKRpSelect, kKRpOut,

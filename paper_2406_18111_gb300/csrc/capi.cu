@@ -131,7 +131,7 @@ ScopeGuard::~ScopeGuard() { c->prof.scope = prev; }
 
 const char *const kKernelNames[kKCount] = {
     "hash_tasks", "init_keys", "key_or", "rs_hist", "rs_offsets", "rs_pass", "refresh", "pack",
-    "phi", "plcp", "lcp_perm", "min32", "max", "cand_gen", "compact", "cand_gather", "greedy",
+    "phi", "plcp", "lcp_perm", "min32", "max", "cand_gen", "compact", "greedy",
     "traces", "sel_out", "pat_layout", "table_init", "end_pairs", "mark_ends", "ac_fix",
     "ac_states", "ac_fill", "dict_insert", "dict_map", "slices", "match_offsets", "seg_scan",
     "starts", "sparse", "ac_nodes", "ac_jump", "rs_tune", "rp_pieces", "rp_need", "rp_chain",
