@@ -768,23 +768,26 @@ struct OpSatSum {
 __global__ void k_flat_chains(const uint4 *__restrict__ rec, const uint32_t *__restrict__ R_dev,
                               const uint32_t *__restrict__ flat_off, const uint32_t *__restrict__ total,
                               const uint32_t *__restrict__ evals, uint32_t P, uint32_t *__restrict__ flat,
-                              uint64_t entries, uint32_t *err) {
-  if (*(volatile uint32_t *)err || *total > entries) return;
-  const uint32_t R = min(P, *R_dev);
+                              uint32_t entries, uint32_t *err) {
+  const uint32_t failed = *(volatile uint32_t *)err, all = *total, R = min(P, *R_dev);
+  if (failed || all > entries) return;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < R; r += warps) {
-    uint64_t o = flat_off[r];
-    uint32_t cur = r;
-    while (cur != kNil) {
-      const uint4 q = cur < R ? rec[cur] : make_uint4(0, 0, kNil, 0);
-      if (q.y == 0 || (uint64_t)q.x + q.y > P || o + q.y > entries) {  // (every record ends a pattern)
+    uint32_t o = flat_off[r];
+    uint4 q = rec[r];
+    while (true) {
+      // (every record ends a pattern, its ids lie in [0, P), the chain ends inside the buffer)
+      const bool bad = (q.y - 1u >= entries - o) | (q.y > P) | (q.x > P - q.y) | ((q.z >= R) & (q.z != kNil));
+      if (bad) {
         if (lane == 0) atomicExch(err, kDevRange);
         break;
       }
+      const uint4 next = q.z != kNil ? rec[q.z] : make_uint4(0, 0, 0, 0);  // under way while the ids are copied
       for (uint32_t k = lane; k < q.y; k += 32) flat[o + k] = evals[q.x + k];
+      if (q.z == kNil) break;
       o += q.y;
-      cur = q.z;
+      q = next;
     }
   }
 }
@@ -1123,17 +1126,21 @@ __global__ void k_lift(const uint32_t *__restrict__ prev_a, uint32_t *__restrict
   }
 }
 
-// Adds the block's matches (v: the lane's) to *total.  64 bits: output places
-// are 32-bit sums, and when the total shows that those wrapped the call fails.
-// One addition per block; called by every warp, with a barrier between the two
-// halves.
+// Adds the block's matches (v: the lane's; sum: the warp's modulo 2^32) to
+// *total.  64 bits: output places are 32-bit sums, and when the total shows
+// that those wrapped the call fails.  One addition per block; called by every
+// warp, with a barrier between the two halves.
 template <int NW>
 struct BlockTotal {
   uint64_t *words;  // [NW] shared
-  __device__ __forceinline__ void put(uint64_t v) {
+  __device__ __forceinline__ void put(uint64_t v, uint32_t sum) {
+    uint64_t w = sum;
+    if (__any_sync(0xffffffffu, v >> 27 != 0)) {  // (otherwise the 32-bit sum is exact)
+      w = v;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = v;
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    }
+    if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = w;
   }
   __device__ __forceinline__ void add(unsigned long long *total) {  // (by warp 1: warp 0 looks back)
     if (threadIdx.x >> 5 != 1) return;
@@ -1176,7 +1183,7 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
     sum = __shfl_sync(0xffffffffu, inc[i], 31);
     mine += v[i];
   }
-  all.put(mine);
+  all.put(mine, sum);
   uint32_t tot;
   const uint32_t ex = scan.run(sum, OpSum(), &tot);
   all.add(matches);
@@ -1200,13 +1207,17 @@ __global__ void __launch_bounds__(kST) k_match_offsets(const uint32_t *__restric
 // I: rows per warp; fewer on short streams, for more tiles.
 // A warp's rows are 32 I consecutive positions: where the matches of a long
 // stream lie on a few of them (256 positions with 4,096 each), the copies of
-// one warp set the time (1.2 ms of 1.9).  Rows of more than kHeavyRow matches
-// are listed instead, and k_match_heavy copies them, a block per row.
+// one warp set the time (1.2 ms of 1.9).  The rows of a warp with more than
+// kHeavyWarp matches are listed instead, and k_match_heavy copies them, a block
+// per row.
 constexpr uint32_t kFillOwn = 4;
-constexpr uint32_t kHeavyRow = 4096;
+constexpr uint32_t kHeavyWarp = 16384;
+constexpr uint32_t kLongChain = 4096;  // of a listed row: copied by the whole block
 constexpr int kFT = 512;
+// Four blocks per SM (32 registers): with 40, three, 2^26 positions 455 us
+// against 375.
 template <int I>
-__global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__ state, uint32_t n,
+__global__ void __launch_bounds__(kFT, 4) k_match_fill(const uint32_t *__restrict__ state, uint32_t n,
                                                     const uint32_t *__restrict__ firstrec,
                                                     const uint32_t *__restrict__ rtot,
                                                     const uint32_t *__restrict__ flat_off,
@@ -1220,8 +1231,12 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
   WarpScan<kFT / 32> scan{s_scan, 0};
   BlockTotal<kFT / 32> all{s_matches};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // (no tile behind an error: the records of an automaton that failed to build mean nothing)
-  if (tid == 0) s_tile = *(volatile uint32_t *)err ? kNil : atomicAdd(tile_ctr, 1u);
+  // (no tile behind an error: the records of an automaton that failed to build
+  // mean nothing; the word is read beside the ticket, not before it)
+  if (tid == 0) {
+    const uint32_t ticket = atomicAdd(tile_ctr, 1u), failed = *(volatile uint32_t *)err;
+    s_tile = failed ? kNil : ticket;
+  }
   __syncthreads();
   if (s_tile == kNil) return;
   const uint32_t t = s_tile;
@@ -1239,7 +1254,7 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
     mine += cnt[i];
   }
   sum = __reduce_add_sync(0xffffffffu, (uint32_t)mine);
-  all.put(mine);
+  all.put(mine, sum);
   uint32_t tot;
   const uint32_t ex = scan.run(sum, OpSum(), &tot);
   all.add(matches);
@@ -1250,17 +1265,21 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
   __syncthreads();
   uint32_t at = s_pre + ex;
   if (sum == 0 || at >= cap) return;  // (the whole warp: no matches, or none that fits)
+  if (sum > kHeavyWarp) {
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      const uint32_t row = __reduce_add_sync(0xffffffffu, cnt[i]);
+      if (lane == 0 && row) heavy[atomicAdd(heavy_n, 1u)] = make_uint2((uint32_t)((seg + i * 32) >> 5), at);
+      at += row;
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < I; ++i) {
     const uint32_t inc = warp_inclusive(cnt[i], OpSum());
-    const uint32_t dst = at + inc - cnt[i], all_row = __shfl_sync(0xffffffffu, inc, 31);
-    if (all_row > kHeavyRow) {
-      if (lane == 0) heavy[atomicAdd(heavy_n, 1u)] = make_uint2((uint32_t)((seg + i * 32) >> 5), at);
-      at += all_row;
-      continue;
-    }
+    const uint32_t dst = at + inc - cnt[i];
     const uint32_t c0 = dst < cap ? (uint32_t)min((uint64_t)cnt[i], cap - dst) : 0u;  // of the chain, what fits
-    at += all_row;
+    at += __shfl_sync(0xffffffffu, inc, 31);
     const uint32_t src = c0 ? flat_off[rec[i]] : 0u;
     const uint32_t x = (uint32_t)(seg + i * 32);
     if (c0 <= kFillOwn) {  // short chains: each lane copies its own
@@ -1282,7 +1301,8 @@ __global__ void __launch_bounds__(kFT) k_match_fill(const uint32_t *__restrict__
 }
 
 // The rows of 32 positions that k_match_fill listed (row, its first output
-// place), when all matches fit: a block per row copies chain after chain.
+// place), when all matches fit: a block per row, a warp per chain, the whole
+// block for a long one.
 __global__ void __launch_bounds__(256) k_match_heavy(const uint2 *__restrict__ heavy, uint32_t rows,
                                                      const uint32_t *__restrict__ state, uint32_t n,
                                                      const uint32_t *__restrict__ firstrec,
@@ -1300,7 +1320,9 @@ __global__ void __launch_bounds__(256) k_match_heavy(const uint2 *__restrict__ h
     for (int j = 0; j < 32; ++j) {  // (every warp holds the row)
       const uint32_t c = __shfl_sync(0xffffffffu, cnt, j), sj = __shfl_sync(0xffffffffu, src, j);
       const uint32_t dj = __shfl_sync(0xffffffffu, dst, j);
-      for (uint32_t k = threadIdx.x; k < c; k += blockDim.x) {
+      const bool own = c < kLongChain;
+      if (own && (uint32_t)j % (blockDim.x / 32) != threadIdx.x / 32) continue;
+      for (uint32_t k = own ? lane : threadIdx.x; k < c; k += own ? 32 : blockDim.x) {
         mend[dj + k] = row.x * 32 + j;
         mid[dj + k] = flat[sj + k];
       }
@@ -1771,7 +1793,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
   const bool early = flat_ok && cap > 0 && P <= n;
   if (early) {
     Launch lp_(c, kKAcFill, P, s);
-    k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, off, n, c->ps.err);
+    k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, off, (uint32_t)n, c->ps.err);
   }
 
   // pass A: the state of every stream position (pass shape chosen above)
@@ -1893,7 +1915,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     uint32_t *side = static_cast<uint32_t *>(c->side);
     {
       Launch lp_(c, kKAcFill, flat_total, s);
-      k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, side, flat_total, c->ps.err);
+      k_flat_chains<<<fblocks, 256, 0, s>>>(rec, R_dev, flat_off, flat_dev, ev, P, side, (uint32_t)flat_total, c->ps.err);
     }
     APO_TRY(fill(side));
     APO_TRY(read_out());

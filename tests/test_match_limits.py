@@ -123,10 +123,13 @@ def test_replay_refuses_more_occurrences_than_31_bits(apo):
 @pytest.mark.parametrize("n,start,k,copies", [(1, 0, 1, 4097), (40, 7, 33, 4096), (5000, 1000, 32, 128),
                                               (5000, 1024, 32, 128), (5000, 1024, 32, 129), (5000, 1010, 32, 300),
                                               (20001, 19993, 8, 9000), ((1 << 22) + 5, 4096, 256, 1000),
-                                              ((1 << 22) + 5, (1 << 22) - 90, 95, 500)])
+                                              ((1 << 22) + 5, (1 << 22) - 90, 95, 500), (3, 1, 1, 20000),
+                                              (5000, 1024, 64, 256), (5000, 1024, 64, 257),
+                                              ((1 << 22) + 5, 4096, 256, 64), ((1 << 22) + 5, 4096, 256, 65)])
 def test_matches_on_few_positions(apo, n, start, k, copies):
-    """k positions with `copies` matches each: rows of 32 positions at and past
-    4,096 matches, cut by the stream's end, in both tile shapes."""
+    """k positions with `copies` matches each: a warp's rows (64 positions, 256 in
+    long streams) at and past 16,384 matches, chains of 4,096 and more, rows cut
+    by the stream's end."""
     import paper_2406_18111_gb300 as gb
     pt, off = nested(copies, 1)
     text = np.full(n, 9, np.uint32)
