@@ -329,7 +329,7 @@ __global__ void k_dict_tokens(const void *__restrict__ tokens, int tb, uint32_t 
   const uint32_t lane = threadIdx.x & 31, lt = lanemask_lt();
   const uint32_t chunk = blockDim.x * kI, chunks = (n + chunk - 1) / chunk;
   for (uint32_t q = blockIdx.x; q < chunks; q += gridDim.x) {
-    const uint64_t b0 = (uint64_t)q * step % chunks * chunk;
+    const uint64_t b0 = (step == 1 ? q : (uint64_t)q * step % chunks) * chunk;
     if (__any_sync(0xffffffffu, *(volatile uint32_t *)over != 0)) break;
     uint64_t t[kI], cur[kI];
     uint32_t fresh = 0;
