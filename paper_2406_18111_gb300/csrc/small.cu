@@ -926,7 +926,7 @@ int read_words(apo_ctx *c, const uint32_t *dev, uint32_t *host, int words, cudaS
 // up to 512 tokens; eight are resident) for 10.3 us + 18.5 ns, u32 tokens 15% less;
 // the general path takes about 750 us + 0.24 ns per token, a little more per token of
 // longer windows.  Windows below 64 tokens, with fewer rounds, cost both sides less:
-// 8.5 us + 47 ns per token here, 450 us + 4.7 us per token there.
+// 8.5 us + 47 ns per token here, 410 us (u64 tokens 470) + 4.7 us per token there.
 // Measured (here / general path, us), u64 tokens, loops with noise and four tokens at
 // random: 10,000 x 64 933 / 1,010 and 834 / 887; 5,000 x 513 1,607 / 1,929 and 1,340 /
 // 1,381; 5,000 x 600 1,671 / 2,051 and 1,395 / 1,486; 10,000 x 1,000 3,862 / 4,751 and
@@ -934,15 +934,16 @@ int read_words(apo_ctx *c, const uint32_t *dev, uint32_t *host, int words, cudaS
 // x 8 678 / 554 and 758 / 522; 20,000 x 128 2,038 / 1,794 and 1,709 / 1,360; 50,000 x
 // 250 5,706 / 5,537 and 4,553 / 3,634; 10,000 x 600 3,196 / 3,232 and 2,669 / 2,226;
 // 50,000 x 513 14,510 / 10,626 and 11,994 / 6,883.
-// What the line costs: loops up to 1.13 times (20,000 x 1,000 u64), random u64 tokens
-// up to 1.7 times.
+// Of 516 batches measured on both sides the line takes the slower one (by 3% or more)
+// for 41: 7 run here, at most 1.08 times slower; given up are loops at up to 1.13 times
+// (20,000 x 1,000 u64) and random u64 tokens at up to 1.7.
 bool small_windows(int sms, uint64_t total, uint64_t windows, uint64_t longest, int token_bytes) {
   if (longest > kSmall[kSmallShapes - 1].max_n) return false;
   const double len = (double)longest;
   const double block = longest > kSmall[0].max_n ? 24.0 + 0.0252 * len
                        : longest >= 64           ? 10.3 + 0.0185 * len
                                                  : 8.5 + 0.047 * len;
-  const double general = longest >= 64 ? 750.0 : 450.0 + 4.7 * len;
+  const double general = longest >= 64 ? 750.0 : (token_bytes == 4 ? 410.0 : 470.0) + 4.7 * len;
   return (double)windows * block * (token_bytes == 4 ? 0.85 : 1.0) / sms <
          general + (0.00024 + 1.3e-8 * len) * (double)total;
 }
