@@ -390,20 +390,24 @@ __device__ __forceinline__ uint32_t block_end(const Sparse &S, uint32_t j, uint3
 // source, length): sorting by it is sorting the pattern strings (disjoint
 // intervals are in string order; a proper prefix has the enclosing interval
 // and sorts first at an equal left end).
+//
+// The arrays are the caller's: what is no permutation is an error (an entry out
+// of range or listed twice; rank[] starts out all-ones), and the kernels behind
+// this one stay inside their arrays and their loops end whatever the entries
+// are -- the host learns of the error only after them.
 __global__ void k_isa(const uint32_t *__restrict__ sa, uint32_t n, uint32_t *__restrict__ rank, uint32_t *err) {
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const uint32_t i = sa[k];
-    if (i < n) rank[i] = k;
-    else atomicExch(err, kDevRange);
+    if (i >= n || atomicExch(&rank[i], k) != kNil) atomicExch(err, kDevRange);
   }
 }
 
 __global__ void k_src_pat_keys(const uint32_t *__restrict__ pstart, const uint32_t *__restrict__ plen, uint32_t P,
-                               const uint32_t *__restrict__ rank, MinTree T, int lenbits, uint64_t *keys,
+                               const uint32_t *__restrict__ rank, uint32_t n, MinTree T, int lenbits, uint64_t *keys,
                                uint32_t *vals, uint32_t *startlen, uint32_t *err) {
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
     const uint32_t st = pstart[p], len = plen[p];
-    const long long j = prev_less(T, rank[st], len, err);
+    const long long j = prev_less(T, min(rank[st], n - 1), len, err);
     keys[p] = ((uint64_t)(j + 1) << lenbits) | len;
     vals[p] = p;
     atomicMax(&startlen[st], len);
@@ -455,9 +459,9 @@ struct OpClampCompose {
 constexpr uint32_t kClampId = 0x0000ffffu;
 struct SrcFnLeft {
   const uint32_t *sa, *lcp, *startlen;
-  uint32_t cap;
+  uint32_t cap, n;
   __device__ __forceinline__ uint32_t operator()(uint32_t k) const {
-    const uint32_t sv = min(startlen[sa[k]], cap), lv = k ? min(lcp[k - 1], cap) : 0u;
+    const uint32_t sv = min(startlen[min(sa[k], n - 1)], cap), lv = k ? min(lcp[k - 1], cap) : 0u;
     return (sv << 16) | lv;
   }
 };
@@ -465,7 +469,7 @@ struct SrcFnRight {
   const uint32_t *sa, *lcp, *startlen;
   uint32_t cap, n;
   __device__ __forceinline__ uint32_t operator()(uint32_t k) const {
-    const uint32_t sv = min(startlen[sa[k]], cap), lv = k + 1 < n ? min(lcp[k], cap) : 0u;
+    const uint32_t sv = min(startlen[min(sa[k], n - 1)], cap), lv = k + 1 < n ? min(lcp[k], cap) : 0u;
     return (sv << 16) | lv;
   }
 };
@@ -475,8 +479,8 @@ struct DstFnLeft {
 };
 struct DstFnRight {  // M of source position SA[k] = the better of both sides
   const uint32_t *sa, *left;
-  uint32_t *mw;
-  __device__ __forceinline__ void operator()(uint32_t k, uint32_t v) const { mw[sa[k]] = max(left[k], v >> 16); }
+  uint32_t *mw, n;
+  __device__ __forceinline__ void operator()(uint32_t k, uint32_t v) const { mw[min(sa[k], n - 1)] = max(left[k], v >> 16); }
 };
 // reach(q) = q + M(q) over T, M(q) = min(the pattern's remaining length,
 // M of the source position), a segment starting at each pattern
@@ -506,6 +510,7 @@ struct NodeArgs {
   // array): failure nodes are found through the source's LCP intervals
   bool src;
   const uint32_t *pstart, *src_rank;
+  uint32_t src_n;
   const uint64_t *skey;  // sorted pattern keys (LCP-interval left end << lenbits | length)
   MinTree T;             // over the source LCP
   int lenbits;
@@ -563,7 +568,7 @@ __global__ void k_ac_nodes(NodeArgs a) {
         if (a.src) {
           // the string's LCP interval in the source; the first pattern in
           // sorted order whose key is not below (left end, fd) starts with it
-          const uint32_t r = a.src_rank[a.pstart[i] + (lo - S)];
+          const uint32_t r = min(a.src_rank[a.pstart[i] + (lo - S)], a.src_n - 1);
           const uint64_t key = ((uint64_t)(prev_less(a.T, r, fd, a.err) + 1) << a.lenbits) | fd;
           uint32_t jl = 0, jh = a.P;
           while (jl < jh) {
@@ -571,8 +576,10 @@ __global__ void k_ac_nodes(NodeArgs a) {
             if (a.skey[mid] < key) jl = mid + 1;
             else jh = mid;
           }
-          if (jl >= a.P) atomicExch(a.err, kDevRange);
-          else f = a.tstart[a.sp[jl]] + fd - 1;
+          const uint32_t q = a.sp[min(jl, a.P - 1)];
+          // (a node of depth fd < d: links always lead up, chains end at the root)
+          if (jl >= a.P || a.plen[q] < fd) atomicExch(a.err, kDevRange);
+          else f = a.tstart[q] + fd - 1;
         } else {
           const uint32_t k = a.rank[lo];
           uint32_t cnt = 0, hi2 = a.P;  // starts before SA index k
@@ -1595,6 +1602,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     // the patterns in string order by their LCP intervals in the source, the
     // start-to-start lcps, and M over the source positions
     const int g = grid_for(src_n, 256, sms);
+    APO_CUDA_TRY(cudaMemsetAsync(src_rank, 0xff, (size_t)src_n * 4, s));
     {
       Launch lp_(c, kKStarts, src_n, s);
       k_isa<<<g, 256, 0, s>>>(pp->src_sa, src_n, src_rank, c->ps.err);
@@ -1603,7 +1611,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     APO_CUDA_TRY(cudaMemsetAsync(startlen, 0, (size_t)src_n * 4, s));
     {
       Launch lp_(c, kKStarts, P, s);
-      k_src_pat_keys<<<grid_for(P, 256, sms), 256, 0, s>>>(pstart, plen, P, src_rank, src_tree, lenbits,
+      k_src_pat_keys<<<grid_for(P, 256, sms), 256, 0, s>>>(pstart, plen, P, src_rank, src_n, src_tree, lenbits,
                                                            b.keys[0], b.vals[0], startlen, c->ps.err);
     }
     b.cur = 0;
@@ -1624,10 +1632,10 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
                                           jpos);
     }
     const uint32_t capv = (uint32_t)maxlen;
-    APO_TRY(seg_scan<false>(c, SrcFnLeft{pp->src_sa, pp->src_lcp, startlen, capv}, DstFnLeft{fl}, src_n,
+    APO_TRY(seg_scan<false>(c, SrcFnLeft{pp->src_sa, pp->src_lcp, startlen, capv, src_n}, DstFnLeft{fl}, src_n,
                             OpClampCompose(), kClampId, s));
     APO_TRY(seg_scan<true>(c, SrcFnRight{pp->src_sa, pp->src_lcp, startlen, capv, src_n},
-                           DstFnRight{pp->src_sa, fl, mw}, src_n, OpClampCompose(), kClampId, s));
+                           DstFnRight{pp->src_sa, fl, mw, src_n}, src_n, OpClampCompose(), kClampId, s));
     APO_TRY(seg_scan<false>(c, SrcReachSrc{tsym, tpid, tstart, plen, pstart, mw}, DstValue{reach}, N,
                             OpSegMax(), kSegMaxId, s));
   } else {
@@ -1722,6 +1730,7 @@ int match_patterns(apo_ctx *c, const apo_patterns *pp, const void *stream, uint6
     a.src = srcm;
     a.pstart = pstart;
     a.src_rank = src_rank;
+    a.src_n = src_n;
     a.skey = skey;
     a.T = src_tree;
     a.lenbits = lenbits;

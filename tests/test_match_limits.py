@@ -1,6 +1,7 @@
 """Matching at its limits: output chains whose flattened length passes 2^32,
 chains longer than the stream, outputs with too little room, more matches
-than 32 bits hold, matches on few positions."""
+than 32 bits hold, matches on few positions, source arrays that are no
+permutation."""
 import ctypes
 
 import numpy as np
@@ -142,3 +143,29 @@ def test_matches_on_few_positions(apo, n, start, k, copies):
         if cap == m:
             assert np.array_equal(e[:m], np.repeat(np.arange(start, start + k, dtype=np.uint32), copies))
             assert np.array_equal(i[:m], np.tile(np.arange(copies, dtype=np.uint32), k))
+
+
+@pytest.mark.parametrize("tb", [4, 8])
+def test_source_array_that_is_no_permutation(apo, tb):
+    """Entries out of range, listed twice, or all the same: APO_EDEVICE, and the
+    context goes on."""
+    import torch
+    import workloads as W
+    from paper_2406_18111_gb300 import ApoError, as_u32
+    S = W.periodic_window(20000, 113, 0.03, 1000, seed=41)
+    t = tokens_dev(S, tb)
+    r = apo.find_repeats(t, 5)
+
+    def match(sa):
+        return apo.match_candidates(t, None, t, pat_start=r.trace_start, pat_len=r.trace_len, src_sa=sa, src_lcp=r.lcp)
+
+    want = match(r.sa)
+    assert len(want[0]) > 1000
+    for at, value in (([0], 20000), ([19999], -1), ([7, 12345], 1 << 30), ([100], int(r.sa[200])),
+                      (list(range(5000)), 17), (list(range(20000)), 0), (list(range(20000)), -2)):
+        bad = r.sa.clone()
+        bad[torch.tensor(at, device="cuda")] = value
+        with pytest.raises(ApoError, match="APO_EDEVICE"):
+            match(bad)
+        got = match(r.sa)
+        assert all(np.array_equal(as_u32(x), as_u32(y)) for x, y in zip(got, want))
