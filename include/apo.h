@@ -575,8 +575,8 @@ int apo_profile_read(apo_ctx *ctx, int index, char *name, size_t name_cap, uint6
  * process (a served lane benefits from another lane's trials); the mode is
  * per context.
  * Results never depend on the shape: the sort is stable and exact.  Calls
- * whose windows are small enough for one block each (at most 8,192 tokens)
- * sort inside the block and tune nothing.
+ * whose windows are small enough for one block each (at most 8,192 tokens, and
+ * not thousands of short ones) sort inside the block and tune nothing.
  * ---------------------------------------------------------------------- */
 int apo_sort_tuning(apo_ctx *ctx, int mode);
 /* Tuned entry `index` (0-based, in class then key-width order): size class

@@ -33,7 +33,7 @@
 // walk in a warp, on those windows at min_len 2: 98,000 with the coverage of
 // the positions ahead as the only bound, 2,900 with the lexicographic bound,
 // 1,800 with the value known as well (both walks counted).  Measured on them:
-// 175 ms before, 6.3 ms with both walks and one warp per block.
+// 175-187 ms before, 5.8-6.4 ms with both walks and one warp per block.
 #include <algorithm>
 #include <vector>
 

@@ -2,7 +2,7 @@
 //
 // A window of a few thousand tokens leaves the many kernels of the general
 // path (suffix.cu, repeats.cu: about 60 launches and six host reads per call)
-// with nothing but their latencies: 590 us for 4,096 tokens of which no
+// with nothing but their latencies: 580-630 us for 4,096 tokens of which no
 // kernel needs more than a few.  Here one launch does every stage of every
 // window, one block each, and the host reads the counts once at the end.  The
 // online finder's slices (250 to 5,000 tokens) and the batches a server forms
@@ -36,8 +36,8 @@
 // barriers; the data never leaves the SM between the stages.  At 4,096 tokens
 // (period 50, 5% noise; 122 us in the kernel): token order 11 us, seven rounds
 // 46, LCP 13, candidates 12, their sort 15, greedy 19, R and outputs 5.
-// Measured per call, before (general path) and now: 4,096 u32 tokens 581 ->
-// 144 us; 40 windows of 250 to 5,000 u64 tokens 810 -> 182 us.
+// Measured per call, before (general path) and now: 4,096 u32 tokens 581-629
+// -> 144-149 us; 40 windows of 250 to 5,000 u64 tokens 830 -> 176-186 us.
 #include <algorithm>
 #include <cstring>
 #include <vector>
