@@ -205,7 +205,7 @@ __global__ void k_slices(const uint32_t *__restrict__ pstart, const uint32_t *__
     const uint32_t l = plen[p];
     if (l == 0) atomicExch(err, kDevRange);
     ml = max(ml, l);
-    me = max(me, pstart[p] + l);
+    me = max(me, pstart[p] + l < l ? 0xffffffffu : pstart[p] + l);  // (an end past 2^32 does not wrap)
     tot += l;
   }
   atomicMax(maxlen, ml);

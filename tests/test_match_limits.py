@@ -169,3 +169,13 @@ def test_source_array_that_is_no_permutation(apo, tb):
             match(bad)
         got = match(r.sa)
         assert all(np.array_equal(as_u32(x), as_u32(y)) for x, y in zip(got, want))
+
+
+@pytest.mark.parametrize("start,length", [((1 << 32) - 1, 2), ((1 << 32) - 5, 5), (1, (1 << 32) - 1)])
+def test_slice_whose_end_wraps(apo, start, length):
+    """A slice that ends past 2^32 is refused (its end, taken modulo 2^32, lies
+    inside the tokens)."""
+    from paper_2406_18111_gb300 import ApoError
+    t = tokens_dev(np.arange(50), 4)
+    with pytest.raises(ApoError, match="APO_EINVAL"):
+        apo.match_candidates(t, None, t, pat_start=tokens_dev([3, start], 4), pat_len=tokens_dev([4, length], 4))
